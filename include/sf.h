@@ -135,7 +135,7 @@ const char *sf_status_str(sf_status s);
  *                   >= 16*chunk slots for chunks up to 65,536, >= 8*chunk above (no
  *                   dictionary with SF_FLAG_SHARED_DICT: see sf_set_dictionary);
  *                   sketches with chunk == 1 and w >= 1024 also hold the one-at-a-time
- *                   dependency-graph workspace (about (16 + 8d) * 512 KiB)
+ *                   workspace of sorts and scans (about (11 + 13d) * 512 KiB)
  * Any output pointer may be NULL.  Returns SF_ERR_INVALID for parameters out of range.
  */
 sf_status sf_required_bytes(const sf_params *p, uint64_t *fat_bytes, uint64_t *slim_bytes,

@@ -11,7 +11,7 @@
 
 #include "sf.h"
 #include "sf_internal.h"
-#include "sf_seqdag.h"
+#include "sf_seqscan.h"
 
 #include "sf_handle.h"
 
@@ -67,9 +67,10 @@ sf_status run_update(sf_sketch* s, const void* keys_in, const int8_t* ops_in, in
         if (staged || st != SF_OK) return st;
     }
     cudaError_t e;
-    if (s->p.chunk == 1 && s->dag_ws && !ops && op_const > 0) {
-        // insertions only: the dependency-graph path (sf_seqdag.cu)
-        e = sfk::launch_seq_dag(desc_of(s), (const uint8_t*)keys, n, s->dag_ws, s->ctrl, s->smem_optin, s->stream);
+    if (s->p.chunk == 1 && s->seq_ws && n > sfk::kSeqScanMinN) {
+        // sorts and scans over pieces of the stream (sf_seqscan.cu)
+        e = sfk::launch_seq_scan(desc_of(s), (const uint8_t*)keys, ops, op_const, n, s->seq_ws, s->ctrl, s->num_sms,
+                                 s->stream);
     } else if (s->p.chunk == 1) {
         sfk::SeqArgs a{};
         a.s = desc_of(s);
@@ -128,9 +129,9 @@ sf_status sf_required_bytes(const sf_params* p, uint64_t* fat_bytes, uint64_t* s
     if (slim_bytes) *slim_bytes = (uint64_t)p->d * p->w * 4ull;
     if (scratch_bytes) {
         const uint64_t cap = (p->chunk > 1 && !(p->flags & SF_FLAG_SHARED_DICT)) ? sfk::dict_capacity(p->chunk) : 0;
-        // S = 1 sketches wide enough for the dependency-graph path also hold its workspace
-        const uint64_t dag = (p->chunk == 1 && sfk::dag_eligible(p->w, p->z)) ? sfk::dag_workspace_bytes(p->d) : 0;
-        *scratch_bytes = kCtrlBytes + cap * sizeof(sfk::DictEntry) + dag;
+        // S = 1 sketches wide enough for the path by sorts and scans also hold its workspace
+        const uint64_t seq = (p->chunk == 1 && sfk::seq_scan_eligible(p->w, p->z)) ? sfk::seq_scan_workspace_bytes(p->d) : 0;
+        *scratch_bytes = kCtrlBytes + cap * sizeof(sfk::DictEntry) + seq;
     }
     return SF_OK;
 }
@@ -170,7 +171,7 @@ sf_status sf_create(const sf_params* p, void* fat_dev, void* slim_dev, void* scr
     s->ctrl = (uint32_t*)scratch_dev;
     s->dict = (p->flags & SF_FLAG_SHARED_DICT) ? nullptr : (sfk::DictEntry*)((uint8_t*)scratch_dev + kCtrlBytes);
     s->cap = p->chunk > 1 ? sfk::dict_capacity(p->chunk) : 0;
-    s->dag_ws = (p->chunk == 1 && sfk::dag_eligible(p->w, p->z)) ? (uint8_t*)scratch_dev + kCtrlBytes : nullptr;
+    s->seq_ws = (p->chunk == 1 && sfk::seq_scan_eligible(p->w, p->z)) ? (uint8_t*)scratch_dev + kCtrlBytes : nullptr;
     sfk::row_seeds(p->seed, p->d, s->rs);
     if (cudaGetDevice(&s->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&s->num_sms, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess ||

@@ -90,7 +90,7 @@ struct sf_sketch {
     uint32_t n_ids;
     uint64_t bar_epoch;     // grid barriers passed on this scratch buffer (monotonic counter)
     uint32_t claims_cap;    // per-block claim list length of the chunk kernel
-    void* dag_ws;           // S = 1 sketches of width >= kDagMinW: workspace of the graph path, else nullptr
+    void* seq_ws;           // S = 1 sketches of width >= kSeqScanMinW: workspace of sf_seqscan.cu, else nullptr
     // Update calls with page-locked host keys stage them through the upper half of the dictionary
     // region (unused by the single-iteration kernel) on a copy stream of their own, created at the
     // first such call.  stage_dirty: that half holds staged bytes, so it is zeroed before a launch

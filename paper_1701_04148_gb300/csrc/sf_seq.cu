@@ -1,4 +1,6 @@
-// sf_seq.cu -- the S = 1 update kernel (sm_103a): the paper's one-at-a-time rule.
+// sf_seq.cu -- the S = 1 update kernel for sketches narrower than 1,024 and for calls of at most 64
+// updates (sm_103a): the paper's one-at-a-time rule in windows of 32 updates.  Longer calls on wider
+// sketches run sf_seqscan.cu.
 //
 // Paper rules (Yang et al., SF-sketch):
 //   insertion (Sec. 3.4, kept by SF_F in Sec. 3.5): B_i[h_i][f_i] += 1 for every row; with

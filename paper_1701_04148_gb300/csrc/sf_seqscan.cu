@@ -1,0 +1,909 @@
+// sf_seqscan.cu -- the paper's one-at-a-time rule (S = 1) by sorts and scans (sm_103a).
+//
+// Rules (Yang et al., SF-sketch): an insertion (Sec. 3.4, kept by SF_F in Sec. 3.5) adds 1 to the
+// item's d Fat counters and then raises its Slim counters to T = min(m + 1, F), where m is the minimum
+// of its Slim counters before and F the minimum of its Fat counters after; a deletion (Sec. 3.5)
+// takes 1 from the Fat counters and lowers A_i[h_i] to M_i = max_k B_i[h_i][k] (SF_4, Sec. 3.4: to the
+// bucket's sum).  The stream is taken in pieces of up to kSeqPiece updates, one cooperative launch
+// each.  What makes a piece parallel:
+//   - A Fat counter's value right after an update is its value before the piece plus the signed count
+//     of the piece's updates on it up to that one: with every row sorted by counter (stable, so stream
+//     order within a counter) a segmented sum.  So every F, and with a search in those sorted rows
+//     every M_i, is known before any Slim counter moves.
+//   - A Slim counter sees, in stream order, x -> max(x, T) at insertions and x -> min(x, M) at
+//     deletions.  Such clamps compose, so with every T known its value before each update is a
+//     segmented scan over the row sorted by bucket.
+//   - Left is T_t = min(m_t + 1, F_t) with m_t depending on earlier T's.  The right side never falls
+//     when a T rises, and m_t reads earlier updates only, so exactly one assignment satisfies it for
+//     every t.  An assignment that an iteration leaves unchanged is therefore the stream-order result.
+//   - From above: T = F everywhere is an upper bound; a scan shows where some row holds less than
+//     T - 1 before the insertion, and T falls to that value plus one.  Sketches whose keys mostly have
+//     one Fat counter to themselves end here at once, or in a few iterations.
+//   - From below, when that does not end soon: every T at first without any other key's raises.  An
+//     iteration follows a key's own raises along the whole piece: on the row sorted by key,
+//     T_j >= min(F_j, 1 + max(a_j, min(T_{j-1}, G_j))), with a_j the key's Slim minimum of the last
+//     iteration and G_j a lower bound of the key's Fat minimum between its updates j - 1 and j (every
+//     clamp M_i in between is at least that).  These maps compose as well (a shift and a clamp), so
+//     this is one more segmented scan.  Dense sketches (z = 1, tens of updates per bucket) take tens of
+//     such iterations; each settles at least the first insertion that is not settled yet.
+//
+// One block of 1,024 threads holds 1,024 consecutive entries of every sorted row, one per thread, in
+// registers across the iterations.  The launch is bound by grid barriers and L2 round trips (about 12
+// barriers when T = F holds), not by bandwidth: its arrays (tens of megabytes at d = 4) stay in L2.
+// Measured on 100,000 Zipf(1) u32 updates (d = 4, w = 4,096, z = 16), a pass: insertions 69 us, where a walk of
+// the stream's dependency graph by one block took 378 us; a tenth of them deletions 121 us, where the
+// window kernel (sf_seq.cu) takes 27.3 ms.
+#include "sf_seqscan.h"
+
+namespace sfk {
+
+namespace {
+
+constexpr uint32_t kTile = 1024;                   // entries of a row per block
+constexpr uint32_t kBlocks = kSeqPiece / kTile;    // blocks of a full piece
+constexpr uint32_t kBins = 256;                    // radix digit of 8 bits
+constexpr uint32_t kGroup = 8;                     // rows ranked at a time (shared memory)
+constexpr uint32_t kAbove = 32;                    // most iterations from above before those from below
+constexpr uint32_t kNear = 16;                     // entries searched back one by one for a key's previous update
+constexpr uint32_t kDirectBlocks = 16;             // up to here every block sums the others' digit counts itself
+constexpr uint32_t kNone = 0xFFFFFFFFu;
+constexpr uint32_t kTop = 0xFFFFFFFFu;
+constexpr uint32_t kOpIns = 1u, kOpDel = 2u;       // operation codes of a sorted element (0: none)
+constexpr uint32_t kHead = 1u << 30, kLast = 1u << 31;
+
+// Workspace of one piece.  A sorted element is key << 32 | position << 2 | operation code, so elements
+// compare by (key, position).  Rows 0..d-1 are sorted by bucket, d..2d-1 by Fat counter (bucket x z +
+// slot), 2d by key hash.
+struct ScanWs {
+    unsigned long long *el0, *el1;  // [2d + 1][N] elements, the two sides of a radix pass
+    ulonglong2* kx;                 // [N] key words by position
+    uint32_t *V, *W, *a;            // [N][row stride] by position: Fat counters after the update; their minima since
+                                    // the key's previous update; Slim counters before the update
+    uint32_t* Vs;                   // [d][N] the Fat counter after the update, in counter order
+    uint32_t *X, *P;                // [N] the raise target; the previous update of the same key
+    uint32_t *hist, *off, *tot;     // digit counts per block (two 16-bit counts a word), first outputs, totals
+    uint4* agg;                     // [d + 1][blocks] block aggregates of a scan
+    uint32_t* low;                  // [d][blocks] least Fat counter of a block's entries in counter order
+    uint32_t* flag;                 // [8] "not settled" and "changed" words of the iterations
+};
+
+__host__ __device__ inline uint32_t rows_of(uint32_t d) { return 2u * d + 1u; }
+
+// Words per position of V, W and a: the rows, so that a thread reads its update's with 16-byte loads.
+__host__ __device__ constexpr uint32_t row_stride(uint32_t d) { return d <= 1 ? 1 : d <= 2 ? 2 : d <= 4 ? 4 : 8; }
+
+__host__ __device__ inline ScanWs carve(void* base, uint32_t d) {
+    const uint64_t N = kSeqPiece, R = rows_of(d);
+    ScanWs w;
+    uint8_t* p = static_cast<uint8_t*>(base);
+    auto take = [&](uint64_t bytes) {
+        uint8_t* q = p;
+        p += (bytes + 255) & ~255ull;
+        return q;
+    };
+    w.el0 = (unsigned long long*)take(R * N * 8);
+    w.el1 = (unsigned long long*)take(R * N * 8);
+    w.kx = (ulonglong2*)take(N * 16);
+    w.V = (uint32_t*)take(row_stride(d) * N * 4);
+    w.W = (uint32_t*)take(row_stride(d) * N * 4);
+    w.a = (uint32_t*)take(row_stride(d) * N * 4);
+    w.Vs = (uint32_t*)take(d * N * 4);
+    w.X = (uint32_t*)take(N * 4);
+    w.P = (uint32_t*)take(N * 4);
+    w.hist = (uint32_t*)take(R * kBlocks * (kBins / 2) * 4);
+    w.off = (uint32_t*)take(R * kBlocks * kBins * 4);
+    w.tot = (uint32_t*)take(R * kBins * 4);
+    w.agg = (uint4*)take((d + 1) * kBlocks * 16);
+    w.low = (uint32_t*)take(d * kBlocks * 4);
+    w.flag = (uint32_t*)take(32);
+    return w;
+}
+
+uint64_t ws_bytes(uint32_t d) {
+    const ScanWs w = carve(nullptr, d);
+    return (uint64_t)(uintptr_t)w.flag + 256;
+}
+
+struct ScanArgs {
+    SketchDesc s;
+    const uint8_t* keys;
+    const int8_t* ops;  // nullptr: every update is op_const
+    int32_t op_const;
+    uint32_t n;         // updates of the piece, at most kSeqPiece
+    uint32_t bucket_passes, counter_passes, key_passes;
+    void* ws;
+    uint32_t* ctrl;
+    uint64_t timeout_ns;
+};
+
+// ---- maps composed by the scans (compose(a, b): first a, then b) -----------------------------
+
+// Segmented sum: y restarts the sum.
+struct SumMap {
+    using T = uint2;  // {sum, restarted}
+    static __device__ __forceinline__ T identity() { return make_uint2(0u, 0u); }
+    static __device__ __forceinline__ T compose(const T& a, const T& b) {
+        return b.y ? b : make_uint2(a.x + b.x, a.y);
+    }
+    static __device__ __forceinline__ T shfl_up(const T& v, int o) {
+        return make_uint2(__shfl_up_sync(kFull, v.x, o), __shfl_up_sync(kFull, v.y, o));
+    }
+    static __device__ __forceinline__ T shfl_down(const T& v, int o) {
+        return make_uint2(__shfl_down_sync(kFull, v.x, o), __shfl_down_sync(kFull, v.y, o));
+    }
+    static __device__ __forceinline__ uint4 pack(const T& v) { return make_uint4(v.x, v.y, 0u, 0u); }
+    static __device__ __forceinline__ T unpack(const uint4& v) { return make_uint2(v.x, v.y); }
+};
+
+// x -> max(lo, min(hi, x)), lo <= hi; a constant when lo = hi.
+struct ClampMap {
+    using T = uint2;  // {lo, hi}
+    static __device__ __forceinline__ T identity() { return make_uint2(0u, kTop); }
+    static __device__ __forceinline__ T compose(const T& a, const T& b) {
+        return make_uint2(max(b.x, min(b.y, a.x)), max(b.x, min(b.y, a.y)));
+    }
+    static __device__ __forceinline__ T shfl_up(const T& v, int o) { return SumMap::shfl_up(v, o); }
+    static __device__ __forceinline__ T shfl_down(const T& v, int o) { return SumMap::shfl_down(v, o); }
+    static __device__ __forceinline__ uint4 pack(const T& v) { return make_uint4(v.x, v.y, 0u, 0u); }
+    static __device__ __forceinline__ T unpack(const uint4& v) { return make_uint2(v.x, v.y); }
+};
+
+__device__ __forceinline__ uint32_t add_sat(uint32_t a, uint32_t b) {
+    const uint32_t s = a + b;
+    return s < a ? kTop : s;
+}
+
+// x -> max(lo, min(hi, x + k)), sums saturating at 2^32 - 1.
+struct ShiftMap {
+    using T = uint3;  // {lo, hi, k}
+    static __device__ __forceinline__ T identity() { return make_uint3(0u, kTop, 0u); }
+    static __device__ __forceinline__ T compose(const T& a, const T& b) {
+        return make_uint3(max(b.x, min(b.y, add_sat(a.x, b.z))), max(b.x, min(b.y, add_sat(a.y, b.z))), a.z + b.z);
+    }
+    static __device__ __forceinline__ T shfl_up(const T& v, int o) {
+        return make_uint3(__shfl_up_sync(kFull, v.x, o), __shfl_up_sync(kFull, v.y, o), __shfl_up_sync(kFull, v.z, o));
+    }
+    static __device__ __forceinline__ T shfl_down(const T& v, int o) {
+        return make_uint3(__shfl_down_sync(kFull, v.x, o), __shfl_down_sync(kFull, v.y, o),
+                          __shfl_down_sync(kFull, v.z, o));
+    }
+    static __device__ __forceinline__ uint4 pack(const T& v) { return make_uint4(v.x, v.y, v.z, 0u); }
+    static __device__ __forceinline__ T unpack(const uint4& v) { return make_uint3(v.x, v.y, v.z); }
+};
+
+// Inclusive scan of the 32 lanes of a warp.
+template <class Map>
+__device__ __forceinline__ typename Map::T warp_scan(typename Map::T v, uint32_t lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const typename Map::T u = Map::shfl_up(v, o);
+        if (lane >= (uint32_t)o) v = Map::compose(u, v);
+    }
+    return v;
+}
+
+struct Shared {
+    union {
+        uint16_t cnt[kGroup][32][kBins];  // digit counts per warp, then first ranks
+        uint32_t part[32][64];            // digit counts of a group of blocks
+        struct {
+            uint32_t V[kMaxD][kTile], pos[kMaxD][kTile], low[kMaxD][32];
+        } tile;
+    } u;
+    uint32_t base[2 * kMaxD + 1][kBins], tot[2 * kMaxD + 1][kBins];
+    uint4 warp_agg[kMaxD][32];
+    uint4 stage[32][32];
+};
+
+// A barrier of the launch's blocks; false: it gave up.
+__device__ __forceinline__ bool piece_barrier(const ScanArgs& a, unsigned long long& target) {
+    if (gridDim.x == 1) {
+        __syncthreads();
+        return true;
+    }
+    const bool ok = grid_barrier(a.ctrl, target, a.timeout_ns);
+    target += gridDim.x;
+    return ok;
+}
+
+// Scan over R rows at once of the whole grid's entries (one per thread and row): v[r] in, the composition
+// of every entry up to and including this one out; prev[r] (if wanted) without it.  One grid barrier.
+// False: the barrier gave up.
+template <class Map, int R, bool kPrev>
+__device__ __forceinline__ bool grid_scan(typename Map::T (&v)[R], typename Map::T (&prev)[R], Shared& sh, uint4* agg,
+                                          const ScanArgs& a, unsigned long long& target) {
+    using T = typename Map::T;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        v[r] = warp_scan<Map>(v[r], lane);
+        if (lane == 31u) sh.warp_agg[r][warp] = Map::pack(v[r]);
+    }
+    __syncthreads();
+    if (warp < (uint32_t)R) {  // warp r: the warps' prefixes of row r, and the block's aggregate
+        const T w = warp_scan<Map>(Map::unpack(sh.warp_agg[warp][lane]), lane);
+        if (lane == 31u) agg[warp * kBlocks + blockIdx.x] = Map::pack(w);
+        T e = Map::shfl_up(w, 1);
+        if (lane == 0u) e = Map::identity();
+        sh.warp_agg[warp][lane] = Map::pack(e);
+    }
+    if (gridDim.x > 1) {
+        if (!grid_barrier(a.ctrl, target, a.timeout_ns)) return false;
+        target += gridDim.x;
+        if (warp < (uint32_t)R && blockIdx.x > 0) {
+            T c = Map::identity();
+#pragma unroll
+            for (uint32_t j = 0; j < kBlocks / 32; ++j) {
+                const uint32_t b = lane * (kBlocks / 32) + j;
+                if (b < blockIdx.x) c = Map::compose(c, Map::unpack(__ldcg(agg + warp * kBlocks + b)));
+            }
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) c = Map::compose(c, Map::shfl_down(c, o));
+            // lane 0 holds the composition of all earlier blocks
+            const uint4 c0 = Map::pack(c);
+            const T carry = Map::unpack(
+                make_uint4(__shfl_sync(kFull, c0.x, 0), __shfl_sync(kFull, c0.y, 0), __shfl_sync(kFull, c0.z, 0), 0u));
+            sh.warp_agg[warp][lane] = Map::pack(Map::compose(carry, Map::unpack(sh.warp_agg[warp][lane])));
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const T before = Map::unpack(sh.warp_agg[r][warp]);
+        if (kPrev) {
+            T e = Map::shfl_up(v[r], 1);
+            if (lane == 0u) e = Map::identity();
+            prev[r] = Map::compose(before, e);
+        }
+        v[r] = Map::compose(before, v[r]);
+    }
+    __syncthreads();  // warp_agg is free again
+    return true;
+}
+
+__device__ __forceinline__ uint32_t el_pos(unsigned long long e) { return ((uint32_t)e >> 2); }
+__device__ __forceinline__ uint32_t el_op(unsigned long long e) { return (uint32_t)e & 3u; }
+__device__ __forceinline__ uint32_t el_key(unsigned long long e) { return (uint32_t)(e >> 32); }
+
+// Stable radix sort, 8 bits a pass, of rows R0..R1-1 (passes(r) passes each; elements start in el0).
+template <int R0, int R1, class Passes>
+__device__ __forceinline__ bool radix_sort(const ScanArgs& a, const ScanWs& w, Shared& sh, unsigned long long& target,
+                                           Passes&& passes_of) {
+    constexpr int R = R1 - R0;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, blk = blockIdx.x;
+    const uint32_t q = blk * kTile + tid;
+    const bool valid = q < a.n;
+    uint32_t passes = 0;
+#pragma unroll
+    for (int r = R0; r < R1; ++r) passes = max(passes, passes_of(r));
+    for (uint32_t p = 0; p < passes; ++p) {
+        const unsigned long long* src = (p & 1u) ? w.el1 : w.el0;
+        unsigned long long* dst = (p & 1u) ? w.el0 : w.el1;
+        uint32_t rk[R];  // rank among the block's equal digits << 8 | digit
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            rk[r] = valid && p < passes_of(R0 + r)
+                        ? (reinterpret_cast<const uint32_t*>(src + (uint64_t)(R0 + r) * kSeqPiece + q)[1] >> (8u * p)) &
+                              (kBins - 1u)
+                        : 0u;
+        const unsigned act = __ballot_sync(kFull, valid);
+        // ranks: the warp's lanes with the same digit from eight ballots (__match_any_sync, which serves the
+        // distinct values one after another, took 2.2 us a row here, the ballots 0.3), then over the
+        // warps in order
+#pragma unroll
+        for (int g = 0; g < R; g += kGroup) {
+#pragma unroll
+            for (int j = 0; j < (int)kGroup && g + j < R; ++j)
+                reinterpret_cast<uint4*>(sh.u.cnt[j][warp])[lane] = make_uint4(0u, 0u, 0u, 0u);
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < (int)kGroup && g + j < R; ++j) {
+                if (p >= passes_of(R0 + g + j)) continue;
+                const uint32_t dig = rk[g + j];
+                unsigned peers = act;
+#pragma unroll
+                for (int b = 0; b < 8; ++b) {
+                    const bool one = (dig >> b) & 1u;
+                    const unsigned m = __ballot_sync(kFull, one);
+                    peers &= one ? m : ~m;
+                }
+                const uint32_t rank = (uint32_t)__popc(peers & ((1u << lane) - 1u));
+                if (valid && rank == 0u) sh.u.cnt[j][warp][dig] = (uint16_t)__popc(peers);
+                rk[g + j] = rank << 8 | dig;
+            }
+            __syncthreads();
+            {
+                const uint32_t j = tid / (kBins / 2), wd = tid % (kBins / 2);  // kGroup rows of 128 words
+                const int r = g + (int)j;
+                if (r < R && p < passes_of(R0 + r)) {
+                    uint32_t run = 0u;  // two 16-bit counts, at most 1,024 each
+#pragma unroll 16
+                    for (uint32_t v = 0; v < 32u; ++v) {
+                        uint32_t* c = reinterpret_cast<uint32_t*>(sh.u.cnt[j][v]) + wd;
+                        const uint32_t x = *c;
+                        *c = run;
+                        run += x;
+                    }
+                    w.hist[((uint32_t)(R0 + r) * kBlocks + blk) * (kBins / 2) + wd] = run;
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < (int)kGroup && g + j < R; ++j) {
+                if (p >= passes_of(R0 + g + j)) continue;
+                rk[g + j] += (uint32_t)sh.u.cnt[j][warp][rk[g + j] & (kBins - 1u)] << 8;
+            }
+            __syncwarp();
+        }
+        if (!piece_barrier(a, target)) return false;
+        // first output of every digit of this block: the same digit of earlier blocks, after all smaller
+        // digits.  A few blocks sum the counts themselves; many share the work, for one more barrier.
+        if (gridDim.x <= kDirectBlocks) {
+            for (uint32_t x = tid; x < (uint32_t)R * (kBins / 2); x += kTile) {
+                const uint32_t r = x / (kBins / 2), wd = x % (kBins / 2);
+                if (p >= passes_of(R0 + (int)r)) continue;
+                uint32_t lo = 0u, hi = 0u, tlo = 0u, thi = 0u;
+                for (uint32_t b = 0; b < gridDim.x; ++b) {
+                    const uint32_t c = __ldcg(w.hist + ((R0 + r) * kBlocks + b) * (kBins / 2) + wd);
+                    if (b == blk) {
+                        lo = tlo;
+                        hi = thi;
+                    }
+                    tlo += c & 0xFFFFu;
+                    thi += c >> 16;
+                }
+                sh.base[r][2 * wd] = lo;
+                sh.base[r][2 * wd + 1] = hi;
+                sh.tot[r][2 * wd] = tlo;
+                sh.tot[r][2 * wd + 1] = thi;
+            }
+        } else {
+            for (uint32_t x = blk; x < (uint32_t)R * 4u; x += gridDim.x) {  // 64 digits of one row
+                const uint32_t r = R0 + (x >> 2), part = x & 3u;
+                if (p >= passes_of((int)r)) continue;
+                constexpr uint32_t kPer = kBlocks / 32;
+                uint32_t lo[kPer], hi[kPer], slo = 0u, shi = 0u;
+#pragma unroll
+                for (uint32_t j = 0; j < kPer; ++j) {
+                    const uint32_t b = warp * kPer + j;
+                    const uint32_t c = b < gridDim.x ? __ldcg(w.hist + (r * kBlocks + b) * (kBins / 2) + part * 32u + lane) : 0u;
+                    lo[j] = slo;
+                    hi[j] = shi;
+                    slo += c & 0xFFFFu;
+                    shi += c >> 16;
+                }
+                sh.u.part[warp][2 * lane] = slo;
+                sh.u.part[warp][2 * lane + 1] = shi;
+                __syncthreads();
+                if (tid < 64u) {
+                    uint32_t run = 0u;
+#pragma unroll 16
+                    for (uint32_t v = 0; v < 32u; ++v) {
+                        const uint32_t y = sh.u.part[v][tid];
+                        sh.u.part[v][tid] = run;
+                        run += y;
+                    }
+                    w.tot[r * kBins + part * 64u + tid] = run;
+                }
+                __syncthreads();
+                const uint32_t blo = sh.u.part[warp][2 * lane], bhi = sh.u.part[warp][2 * lane + 1];
+#pragma unroll
+                for (uint32_t j = 0; j < kPer; ++j) {
+                    const uint32_t b = warp * kPer + j;
+                    if (b < gridDim.x)
+                        *reinterpret_cast<uint2*>(w.off + (r * kBlocks + b) * kBins + part * 64u + 2 * lane) =
+                            make_uint2(blo + lo[j], bhi + hi[j]);
+                }
+                __syncthreads();
+            }
+            if (!piece_barrier(a, target)) return false;
+            for (uint32_t x = tid; x < (uint32_t)R * kBins; x += kTile) {
+                const uint32_t r = x / kBins, b = x % kBins;
+                if (p >= passes_of(R0 + (int)r)) continue;
+                sh.base[r][b] = __ldcg(w.off + ((R0 + r) * kBlocks + blk) * kBins + b);
+                sh.tot[r][b] = __ldcg(w.tot + (R0 + r) * kBins + b);
+            }
+        }
+        __syncthreads();
+        for (uint32_t r = warp; r < (uint32_t)R; r += 32u) {  // digits of a row: exclusive scan of the totals
+            if (p >= passes_of(R0 + (int)r)) continue;
+            uint32_t c[8], sum = 0u;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                c[j] = sum;
+                sum += sh.tot[r][lane * 8u + j];
+            }
+            uint32_t incl = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= (uint32_t)o) incl += y;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sh.base[r][lane * 8u + j] += incl - sum + c[j];
+        }
+        __syncthreads();
+        if (valid) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (p < passes_of(R0 + r))
+                    dst[(uint64_t)(R0 + r) * kSeqPiece + sh.base[r][rk[r] & (kBins - 1u)] + (rk[r] >> 8)] =
+                        src[(uint64_t)(R0 + r) * kSeqPiece + q];
+        }
+        if (!piece_barrier(a, target)) return false;
+    }
+    return true;
+}
+
+// kIns: the piece holds insertions only; kDel: deletions only.
+template <int D, bool kIns, bool kDel>
+__global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constant__ ScanArgs a) {
+    constexpr uint32_t kStride = row_stride(D);
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    Shared& sh = *reinterpret_cast<Shared*>(s_raw);
+    const SketchDesc& s = a.s;
+    const ScanWs w = carve(a.ws, D);
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, blk = blockIdx.x;
+    const uint32_t q = blk * kTile + tid;  // this thread's position, and its index in every sorted row
+    const bool valid = q < a.n;
+    const uint32_t wz = s.w * s.z;
+    unsigned long long target = gridDim.x;
+    auto barrier = [&]() { return piece_barrier(a, target); };
+
+    // ---- hash --------------------------------------------------------------------------------
+    {
+        const uint32_t kb = s.key_bytes;
+        const uint32_t first = blk * kTile + warp * 32u;
+        const uint32_t nv = first < a.n ? min(32u, a.n - first) : 0u;
+        Key k{0ull, 0ull};
+        if (kb != 4u && kb != 8u) {
+            if (nv) k = load_key_staged(a.keys, (uint64_t)a.n * kb, first, nv, kb, lane, sh.stage[warp]);
+        } else if (valid) {
+            k = load_key(a.keys, q, kb);
+        }
+        uint32_t h[D], f[D], op = 0u;
+        uint64_t probe = 0;
+#pragma unroll
+        for (int i = 0; i < D; ++i) h[i] = f[i] = 0u;
+        if (valid) {
+            const int o = a.ops ? (int)a.ops[q] : a.op_const;
+            op = o > 0 ? kOpIns : o < 0 ? kOpDel : 0u;
+            if (op && !key_indices<D>(s, k, h, f, &probe)) {
+                atomicOr(a.ctrl + kCtrlErr, kErrBadKey);
+                op = 0u;
+#pragma unroll
+                for (int i = 0; i < D; ++i) h[i] = f[i] = 0u;  // does nothing, in bucket 0
+            }
+        }
+        const uint32_t pay = q << 2 | op;
+        const uint32_t tag = (uint32_t)(probe >> 32) * 0x9E3779B1u ^ (uint32_t)probe;
+        if (valid) {
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                w.el0[(uint64_t)i * kSeqPiece + q] = (unsigned long long)h[i] << 32 | pay;
+                w.el0[(uint64_t)(D + i) * kSeqPiece + q] = (unsigned long long)(h[i] * s.z + f[i]) << 32 | pay;
+            }
+            if constexpr (!kDel) {
+                w.el0[(uint64_t)(2 * D) * kSeqPiece + q] =
+                    (unsigned long long)(tag >> (32u - 8u * a.key_passes)) << 32 | pay;
+                w.kx[q] = make_ulonglong2(k.x0, k.x1);
+            }
+        }
+        if (blk == 0 && tid < 8u) w.flag[tid] = 0u;
+    }
+
+    // ---- sort by bucket and by Fat counter -----------------------------------------------------------
+    if (!radix_sort<0, 2 * D>(a, w, sh, target, [&](int r) { return r < D ? a.bucket_passes : a.counter_passes; })) return;
+    auto row = [&](int r) {  // the sorted row
+        const uint32_t passes = r < D ? a.bucket_passes : r < 2 * D ? a.counter_passes : a.key_passes;
+        return ((passes & 1u) ? w.el1 : w.el0) + (uint64_t)r * kSeqPiece;
+    };
+
+    // ---- Fat counters after every update -------------------------------------------------------------
+    {
+        uint2 v[D], unused[D];
+        uint32_t po[D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            v[i] = SumMap::identity();
+            po[i] = 0u;
+            if (valid) {
+                const unsigned long long* C = row(D + i);
+                const unsigned long long e = C[q];
+                const uint32_t key = el_key(e), op = el_op(e);
+                const bool head = q == 0u || el_key(C[q - 1u]) != key;
+                po[i] = (uint32_t)e;
+                v[i].x = op == kOpIns ? 1u : op == kOpDel ? kTop : 0u;
+                if (head) {
+                    v[i].x += __ldcg(s.B + (uint64_t)i * wz + key);
+                    v[i].y = 1u;
+                }
+            }
+        }
+        if (!grid_scan<SumMap, D, false>(v, unused, sh, w.agg, a, target)) return;
+        bool under = false;
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            if (!valid) continue;
+            w.V[(uint64_t)(po[i] >> 2) * kStride + i] = v[i].x;
+            w.Vs[(uint64_t)i * kSeqPiece + q] = v[i].x;
+            under |= (po[i] & 3u) == kOpDel && v[i].x == kTop;
+        }
+        if (under) atomicOr(a.ctrl + kCtrlErr, kErrUnderflow);
+    }
+    if (!barrier()) return;
+
+    // ---- this thread's entries of the bucket orders; deletions find their bounds ----------------------
+    uint32_t bpo[D], M[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        bpo[i] = 0u;
+        M[i] = 0u;
+        const unsigned long long* Bo = row(i);
+        uint32_t h = 0u;
+        if (valid) {
+            const unsigned long long e = Bo[q];
+            h = el_key(e);
+            bpo[i] = (uint32_t)e;
+            if (q == 0u || el_key(Bo[q - 1u]) != h) bpo[i] |= kHead;
+            if (q + 1u == a.n || el_key(Bo[q + 1u]) != h) bpo[i] |= kLast;
+        }
+        if constexpr (!kIns) {
+            // M_i: the bucket's counters right after the deletion, each by a binary search for the last
+            // update on it up to the deletion; a group of lanes takes a deletion, a lane its counters
+            // (the bucket's entries take the same places in both orders, so a bucket that begins and ends
+            // inside this block is searched alone: about 5 steps instead of 17 for 24 entries)
+            const uint32_t gl = s.z <= 4u ? 4u : s.z <= 8u ? 8u : s.z <= 16u ? 16u : 32u;
+            const unsigned long long* C = row(D + i);
+            const unsigned heads = __ballot_sync(kFull, (bpo[i] & kHead) != 0u);
+            if (lane == 0u) sh.tot[i][warp] = heads;
+            __syncthreads();
+            uint32_t first = 0u, end = a.n;
+            if ((bpo[i] & 3u) == kOpDel) {
+                unsigned b = heads & (kTop >> (31u - lane));
+                int wv = (int)warp;
+                while (!b && wv > 0) b = sh.tot[i][--wv];
+                if (b) first = blk * kTile + (uint32_t)wv * 32u + 31u - (uint32_t)__clz(b);
+                b = lane == 31u ? 0u : heads & (kTop << (lane + 1u));
+                wv = (int)warp;
+                while (!b && wv < 31) b = sh.tot[i][++wv];
+                if (b) end = blk * kTile + (uint32_t)wv * 32u + (uint32_t)__ffs(b) - 1u;
+            }
+            unsigned todo = __ballot_sync(kFull, (bpo[i] & 3u) == kOpDel);
+            while (todo) {
+                // the group's deletion: the (lane / gl)-th lane of todo that still waits
+                unsigned rest = todo;
+                for (uint32_t g = 0; g < lane / gl && rest; ++g) rest &= rest - 1u;
+                const int from = rest ? __ffs(rest) - 1 : -1;
+                const uint32_t hd = __shfl_sync(kFull, h, from < 0 ? 0 : from);
+                const uint32_t pd = __shfl_sync(kFull, bpo[i], from < 0 ? 0 : from) & ~(kHead | kLast);
+                const uint32_t f0 = __shfl_sync(kFull, first, from < 0 ? 0 : from);
+                const uint32_t f1 = __shfl_sync(kFull, end, from < 0 ? 0 : from);
+                uint32_t mx = 0u;
+                uint64_t sum = 0ull;
+                if (from >= 0) {
+                    for (uint32_t k = lane % gl; k < s.z; k += gl) {
+                        const uint32_t key = hd * s.z + k;
+                        const unsigned long long want = (unsigned long long)key << 32 | pd | 3u;
+                        uint32_t lo = f0, hi = f1;  // entries below lo are <= want, from hi on > want
+                        while (lo < hi) {
+                            const uint32_t mid = (lo + hi) >> 1;
+                            if (C[mid] <= want) lo = mid + 1u;
+                            else hi = mid;
+                        }
+                        const bool hit = lo > 0u && el_key(C[lo - 1u]) == key;
+                        const uint32_t v = hit ? w.Vs[(uint64_t)i * kSeqPiece + lo - 1u]
+                                               : __ldcg(s.B + (uint64_t)i * wz + key);
+                        mx = max(mx, v);
+                        sum += v;
+                    }
+                }
+                for (uint32_t o = gl >> 1; o > 0u; o >>= 1) {
+                    mx = max(mx, __shfl_xor_sync(kFull, mx, o));
+                    sum += __shfl_xor_sync(kFull, sum, o);
+                }
+                const uint32_t bound = s.sf4_delete ? (sum < (uint64_t)kTop ? (uint32_t)sum : kTop) : mx;
+                // hand the bounds back and strike the deletions taken
+                for (uint32_t g = 0; g < 32u / gl && todo; ++g) {
+                    const int at = __ffs(todo) - 1;
+                    const uint32_t b = __shfl_sync(kFull, bound, g * gl);
+                    if ((int)lane == at) M[i] = b;
+                    todo &= todo - 1u;
+                }
+            }
+        }
+    }
+
+    auto least_of = [&](const uint32_t* by_pos, uint32_t pos) {  // minimum over the rows at a position
+        uint32_t v[kStride], m = kTop;
+        if constexpr (kStride >= 4u) {
+#pragma unroll
+            for (uint32_t j = 0; j < kStride; j += 4u)
+                *reinterpret_cast<uint4*>(v + j) = __ldcg(reinterpret_cast<const uint4*>(by_pos + (uint64_t)pos * kStride + j));
+        } else {
+#pragma unroll
+            for (uint32_t j = 0; j < kStride; ++j) v[j] = __ldcg(by_pos + (uint64_t)pos * kStride + j);
+        }
+#pragma unroll
+        for (int i = 0; i < D; ++i) m = min(m, v[i]);
+        return m;
+    };
+
+    // Slim counters along the bucket orders with raise targets T[i] of this thread's entries: v[i].x after
+    // an entry, prev[i].x before it.
+    uint2 v[D], prev[D];
+    auto slim_scan = [&](const uint32_t (&T)[D]) -> bool {
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            const uint32_t op = bpo[i] & 3u;
+            v[i] = op == kOpIns ? make_uint2(T[i], kTop) : op == kOpDel ? make_uint2(0u, M[i]) : ClampMap::identity();
+            if (bpo[i] & kHead) {
+                const uint32_t A0 = __ldcg(slim_ptr(s, i, el_key(row(i)[q])));
+                const uint32_t x = max(v[i].x, min(v[i].y, A0));
+                v[i] = make_uint2(x, x);
+            }
+        }
+        if (!grid_scan<ClampMap, D, true>(v, prev, sh, w.agg, a, target)) return false;
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+            if (bpo[i] & kHead) prev[i].x = __ldcg(slim_ptr(s, i, el_key(row(i)[q])));
+        return true;
+    };
+    auto pos_of = [&](int i) { return (bpo[i] & ~(kHead | kLast)) >> 2; };
+    // How many threads of the grid say yes: the words of w.flag rotate over four, and each is cleared two
+    // calls before its next use.  One grid barrier; kNone: it gave up.
+    uint32_t calls = 0;
+    auto count_of_grid = [&](bool mine) -> uint32_t {
+        const uint32_t word = calls & 3u;
+        if (blk == 0u && tid == 0u) w.flag[(calls + 2u) & 3u] = 0u;
+        ++calls;
+        const uint32_t c = (uint32_t)__syncthreads_count(mine);
+        if (c && tid == 0u) atomicAdd(w.flag + word, c);
+        if (!barrier()) return kNone;
+        return __ldcg(w.flag + word);
+    };
+
+    uint32_t T[D];
+    bool settled = true;
+    if constexpr (kDel) {
+#pragma unroll
+        for (int i = 0; i < D; ++i) T[i] = 0u;
+        if (!slim_scan(T)) return;
+    } else {
+        // ---- raise targets from above: T = F, lowered where a row holds less than T - 1 ------------------
+        if (valid) w.X[q] = least_of(w.V, q);
+        uint32_t most = a.n / 16u;
+        for (uint32_t it = 0;; ++it) {
+#pragma unroll
+            for (int i = 0; i < D; ++i)
+                T[i] = (bpo[i] & 3u) != kOpIns ? 0u : it == 0u ? least_of(w.V, pos_of(i)) : __ldcg(w.X + pos_of(i));
+            if (!slim_scan(T)) return;
+            bool lower = false;
+#pragma unroll
+            for (int i = 0; i < D; ++i)
+                if ((bpo[i] & 3u) == kOpIns && prev[i].x < T[i] && prev[i].x + 1u < T[i]) {
+                    atomicMin(w.X + pos_of(i), prev[i].x + 1u);
+                    lower = true;
+                }
+            const uint32_t more = count_of_grid(lower);
+            if (more == kNone) return;
+            settled = more == 0u;
+            // Go on while the count falls fast: on streams with few coupled keys it falls to a third or less
+            // an iteration, on dense sketches by a tenth.  An iteration takes 8 us at d = 4, the way from
+            // below 20 us before its first one and 12 us for each.
+            if (settled || it == kAbove || (more > 4u && 8u * more > 5u * most)) break;
+            most = more;
+        }
+    }
+    if constexpr (!kDel) {
+        if (!settled) {
+            // ---- from below: the rows in key order, and each entry's previous update of its key ----------
+            if (!radix_sort<2 * D, 2 * D + 1>(a, w, sh, target, [&](int) { return a.key_passes; })) return;
+            uint32_t kpo = 0u;  // this thread's entry: position << 2 | operation, kHead
+            if (valid) {
+                const unsigned long long* K = row(2 * D);
+                const unsigned long long e = K[q];
+                const uint32_t pos = el_pos(e);
+                uint32_t before = kNone;
+                if (q > 0u) {
+                    const unsigned long long b = K[q - 1u];
+                    if (el_key(b) == el_key(e)) {
+                        const ulonglong2 x = w.kx[pos], y = w.kx[el_pos(b)];
+                        if (x.x == y.x && x.y == y.y && el_op(e) && el_op(b)) before = el_pos(b);
+                    }
+                }
+                kpo = (uint32_t)e | (before == kNone ? kHead : 0u);
+                w.P[pos] = before;
+            }
+            if constexpr (!kIns) {
+                // W: a lower bound of the counter's least value since the key's previous update, from the
+                // entries before this one in counter order until the previous update is covered: at least
+                // kNear one by one, then whole warps' and whole blocks' least values (which may hold
+                // entries of another counter, or of before the previous update: lower at worst)
+#pragma unroll
+                for (int i = 0; i < D; ++i) {
+                    const uint32_t x = valid ? w.Vs[(uint64_t)i * kSeqPiece + q] : kTop;
+                    sh.u.tile.V[i][tid] = x;
+                    sh.u.tile.pos[i][tid] = valid ? el_pos(row(D + i)[q]) : kNone;
+                    const uint32_t l = __reduce_min_sync(kFull, x);
+                    if (lane == 0u) sh.u.tile.low[i][warp] = l;
+                }
+                __syncthreads();
+                if (tid < 32u) {
+#pragma unroll
+                    for (int i = 0; i < D; ++i) {
+                        const uint32_t l = __reduce_min_sync(kFull, sh.u.tile.low[i][tid]);
+                        if (tid == 0u) w.low[i * kBlocks + blk] = l;
+                    }
+                }
+                if (!barrier()) return;
+#pragma unroll
+                for (int i = 0; i < D; ++i) {
+                    if (!valid) continue;
+                    const uint32_t pos = sh.u.tile.pos[i][tid], target_pos = w.P[pos];
+                    uint32_t least = kTop;
+                    if (target_pos != kNone) {
+                        bool found = false;
+                        uint32_t j = q;  // the entries from j on have been looked at
+                        for (uint32_t c = 0; !found && j > 0u && (c < kNear || (j & 31u) != 0u); ++c) {
+                            --j;
+                            const bool here = j >= blk * kTile;
+                            least = min(least, here ? sh.u.tile.V[i][j - blk * kTile]
+                                                    : __ldcg(w.Vs + (uint64_t)i * kSeqPiece + j));
+                            found = (here ? sh.u.tile.pos[i][j - blk * kTile] : el_pos(row(D + i)[j])) == target_pos;
+                        }
+                        // A warp or block is passed whole while its first entry is a later update of this
+                        // counter.  Where its first entry is on another counter, the counter's entries
+                        // begin inside it, so the previous update lies inside it or was passed.
+                        while (!found && j > blk * kTile) {
+                            j -= 32u;
+                            least = min(least, sh.u.tile.low[i][(j - blk * kTile) / 32u]);
+                            found = sh.u.tile.pos[i][j - blk * kTile] <= target_pos;
+                        }
+                        for (uint32_t b = (j + kTile - 1u) / kTile; !found && b-- > 0u;) {
+                            least = min(least, __ldcg(w.low + i * kBlocks + b));
+                            found = el_pos(row(D + i)[b * kTile]) <= target_pos;
+                        }
+                    }
+                    w.W[(uint64_t)pos * kStride + i] = least;
+                }
+            }
+            const uint32_t kop = kpo & 3u, kpos = (kpo & ~kHead) >> 2;
+            uint32_t F = kTop, G = kTop, x = 0u;
+            if (valid) F = least_of(w.V, kpos);
+            // at most one iteration per update: each settles at least the first unsettled insertion
+            for (uint32_t it = 0; it <= a.n; ++it) {
+#pragma unroll
+                for (int i = 0; i < D; ++i)
+                    T[i] = (bpo[i] & 3u) == kOpIns && it > 0u ? __ldcg(w.X + pos_of(i)) : 0u;
+                if (!slim_scan(T)) return;
+#pragma unroll
+                for (int i = 0; i < D; ++i)
+                    if ((bpo[i] & 3u) == kOpIns) w.a[(uint64_t)pos_of(i) * kStride + i] = prev[i].x;
+                if (!barrier()) return;
+                uint3 f[1], unused[1];
+                f[0] = ShiftMap::identity();
+                if (valid) {
+                    if (kop == kOpIns) {
+                        const uint32_t m = least_of(w.a, kpos);
+                        if constexpr (!kIns)
+                            if (it == 0u) G = least_of(w.W, kpos);
+                        const uint32_t lo = min(F, add_sat(m, 1u));
+                        f[0] = (kpo & kHead) ? make_uint3(lo, lo, 0u)
+                                             : make_uint3(lo, min(F, add_sat(max(m, G), 1u)), 1u);
+                    } else if (kpo & kHead) {
+                        f[0] = make_uint3(0u, 0u, 0u);  // nothing known of the key's Slim minimum yet
+                    } else {
+                        if constexpr (!kIns)
+                            if (it == 0u) G = least_of(w.W, kpos);
+                        f[0] = make_uint3(0u, min(G, F), 0u);  // a deletion
+                    }
+                }
+                if (!grid_scan<ShiftMap, 1, false>(f, unused, sh, w.agg + (uint64_t)D * kBlocks, a, target)) return;
+                bool changed = false;
+                if (valid && kop == kOpIns) {
+                    changed = it == 0u || f[0].x != x;
+                    x = f[0].x;
+                    w.X[kpos] = x;
+                }
+                const uint32_t more = count_of_grid(changed);
+                if (more == kNone) return;
+                if (more == 0u) break;  // X is as before this iteration, so v holds the counters after it
+            }
+        }
+    }
+
+    // ---- the counters after the piece ------------------------------------------------------------------
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        if (bpo[i] & kLast) *slim_ptr(s, i, el_key(row(i)[q])) = v[i].x;
+        if (valid) {
+            const unsigned long long* C = row(D + i);
+            const uint32_t key = el_key(C[q]);
+            if (q + 1u == a.n || el_key(C[q + 1u]) != key)
+                s.B[(uint64_t)i * wz + key] = w.Vs[(uint64_t)i * kSeqPiece + q];
+        }
+    }
+    // the last block to leave resets the barrier for the next launch
+    if (tid == 0u && gridDim.x > 1u) {
+        if (atomicAdd(a.ctrl + kCtrlSeqDone, 1u) == gridDim.x - 1u) {
+            *reinterpret_cast<unsigned long long*>(a.ctrl + kCtrlBarrier64) = 0ull;
+            a.ctrl[kCtrlSeqDone] = 0u;
+        }
+    }
+}
+
+template <int D, bool kIns, bool kDel>
+cudaError_t launch_kind(const ScanArgs& a, uint32_t blocks, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(seq_scan_kernel<D, kIns, kDel>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(Shared));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kTile);
+    cfg.dynamicSmemBytes = sizeof(Shared);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, seq_scan_kernel<D, kIns, kDel>, a);
+}
+
+template <int D>
+cudaError_t launch_d(const ScanArgs& a, uint32_t blocks, cudaStream_t st) {
+    if (a.ops) return launch_kind<D, false, false>(a, blocks, st);
+    if (a.op_const > 0) return launch_kind<D, true, false>(a, blocks, st);
+    return launch_kind<D, false, true>(a, blocks, st);
+}
+
+uint32_t digits_of(uint64_t limit) {  // 8-bit digits of keys below limit
+    uint32_t p = 1;
+    while (p < 4 && ((limit - 1) >> (8 * p)) != 0) ++p;
+    return p;
+}
+
+}  // namespace
+
+uint64_t seq_scan_workspace_bytes(uint32_t d) { return ws_bytes(d); }
+
+cudaError_t launch_seq_scan(const SketchDesc& s, const uint8_t* keys, const int8_t* ops, int32_t op_const, uint64_t n,
+                            void* ws, uint32_t* ctrl, int num_sms, cudaStream_t st) {
+    const uint64_t wz = (uint64_t)s.w * s.z;
+    if (wz >= (1ull << 32)) return cudaErrorInvalidValue;
+    // every block of a launch must be resident: one per SM
+    const uint64_t most = (uint64_t)num_sms * kTile;
+    const uint64_t piece = most < kSeqPiece ? most : kSeqPiece;
+    for (uint64_t base = 0; base < n; base += piece) {
+        ScanArgs a{};
+        a.s = s;
+        a.keys = keys + base * s.key_bytes;
+        a.ops = ops ? ops + base : nullptr;
+        a.op_const = op_const;
+        a.n = (uint32_t)(n - base < piece ? n - base : piece);
+        a.bucket_passes = digits_of(s.w);
+        a.counter_passes = digits_of(wz);
+        a.key_passes = a.n <= 2048u ? 2u : 3u;
+        a.ws = ws;
+        a.ctrl = ctrl;
+        a.timeout_ns = kBarrierTimeoutNs;
+        const uint32_t blocks = (a.n + kTile - 1) / kTile;
+        cudaError_t e = cudaErrorInvalidValue;
+        switch (s.d) {
+            case 1: e = launch_d<1>(a, blocks, st); break;
+            case 2: e = launch_d<2>(a, blocks, st); break;
+            case 3: e = launch_d<3>(a, blocks, st); break;
+            case 4: e = launch_d<4>(a, blocks, st); break;
+            case 5: e = launch_d<5>(a, blocks, st); break;
+            case 6: e = launch_d<6>(a, blocks, st); break;
+            case 7: e = launch_d<7>(a, blocks, st); break;
+            case 8: e = launch_d<8>(a, blocks, st); break;
+            default: break;
+        }
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace sfk

@@ -25,7 +25,7 @@
 // T_e <= F_e <= that bound, so the raises and clamps of a
 // counter commute: applying them with atomics in any order gives the stream-order result.
 //
-// The S = 1 path (the paper's one-at-a-time rule) is seq_update_kernel in sf_seq.cu.
+// The S = 1 path (the paper's one-at-a-time rule) is in sf_seqscan.cu and sf_seq.cu.
 #pragma once
 
 #include "sf_internal.h"
