@@ -14,7 +14,7 @@
 struct sf_batch {
     uint32_t max_sketches;
     uint64_t max_round_slots;
-    uint2* claims_dev;
+    uint4* claims_dev;
     uint8_t* scratch;
     uint32_t* ctrl;
     sfk::SketchRun* table_dev;
@@ -116,7 +116,7 @@ sf_status sf_batch_create(uint32_t max_sketches, uint64_t max_round_slots, void*
         delete b;
         return SF_ERR_OOM;
     }
-    b->claims_dev = (uint2*)((uint8_t*)scratch_dev + kBatchCtrlBytes + table_bytes_of(max_sketches));
+    b->claims_dev = (uint4*)((uint8_t*)scratch_dev + kBatchCtrlBytes + table_bytes_of(max_sketches));
     b->scratch = (uint8_t*)scratch_dev;
     b->ctrl = (uint32_t*)scratch_dev;
     b->table_dev = (sfk::SketchRun*)((uint8_t*)scratch_dev + kBatchCtrlBytes);
@@ -308,7 +308,7 @@ sf_status sf_batch_update(sf_batch* b, uint32_t n_items, const sf_batch_item* it
         a.keys_in_host = in_host ? 1 : 0;
         // claim lists in shared memory when they fit, else in the batch scratch (launches run in order)
         a.claims_global =
-            ((uint64_t)a.claims_cap * sizeof(uint2) > (uint64_t)sfk::claim_smem_max(block)) ? b->claims_dev : nullptr;
+            ((uint64_t)a.claims_cap * sizeof(uint4) > (uint64_t)sfk::claim_smem_max(block)) ? b->claims_dev : nullptr;
         b->plan.push_back(a);
         rounds_all = rounds > rounds_all ? rounds : rounds_all;
     }

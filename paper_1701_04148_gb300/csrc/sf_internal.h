@@ -32,10 +32,11 @@ struct BatchArgs {
     uint64_t n_rounds;      // max over sketches of ceil(n / S)
     uint32_t* ctrl;         // error word + barrier counter
     uint64_t bar_base;      // grid barriers the counter has passed before this launch
+    uint32_t arrive;        // what a block adds to the counter at a barrier (set by the launch)
     uint64_t timeout_ns;
     int32_t may_ins;        // some update of the launch may be an insertion
     int32_t may_del;        // ... a deletion
-    uint2* claims_global;   // per-block claim lists in global memory (claims_cap each), or nullptr: shared memory
+    uint4* claims_global;   // per-block claim lists in global memory (claims_cap each), or nullptr: shared memory
     uint32_t max_chunk;     // largest S of the launch's sketches
     int32_t keys_in_host;   // some sketch's keys (or operations) live in host memory, read over the host link
 };
@@ -100,7 +101,13 @@ constexpr int kChunkBlock = 512;  // default block of the chunked-update kernels
 constexpr int kSeqBlock = 256;
 constexpr int kQueryBlock = 256;
 constexpr uint64_t kBarrierTimeoutNs = 2000000000ull;  // 2 s per wait
-constexpr int kMaxClaimSmem = 96 * 1024;               // dynamic shared memory for the claim list
+constexpr int kMaxClaimSmem = 112 * 1024;              // dynamic shared memory for the claim list: 7,168 claims of 16
+                                                       // bytes, a block's share of a 2^20-update chunk over 147 SMs or
+                                                       // more; batches keep longer lists in their scratch
+constexpr int kMostClaimSmem = 160 * 1024;             // up to here a launch of one sketch may go: 103 SMs
+// The barrier counter is kept across launches whose grids differ by a factor of two (the multi-iteration
+// kernel runs two blocks where the others run one): a barrier adds kArriveUnits x the smaller grid.
+constexpr uint32_t kArriveUnits = 2;
 
 // Chunked update: one cooperative persistent launch per call (one sketch or a batch of sketches
 // sharing d) of `grid` blocks of `block` threads (512, 256 or 128); 2 grid barriers per round.
@@ -110,12 +117,12 @@ template <int B>
 cudaError_t launch_batch_block(const BatchArgs& a, uint32_t d, int grid, cudaStream_t st);
 template <int B>
 int blocks_per_sm_block(uint32_t d);
-// Dynamic shared memory a block may use for its claim list: 96 KiB at 512 threads, in proportion
+// Dynamic shared memory a block may use for its claim list: 112 KiB at 512 threads, in proportion
 // below, so that 512 / block blocks of a launch fit one SM.
 inline int claim_smem_max(int block) { return kMaxClaimSmem * block / kChunkBlock; }
 // Global claim-list bytes a launch over rounds of up to max_round_slots slots may need (any grid <= 1024 blocks).
 inline uint64_t claims_global_bytes(uint64_t max_round_slots) {
-    return (max_round_slots + 1024ull * kChunkBlock) * 8ull;
+    return (max_round_slots + 1024ull * kChunkBlock) * sizeof(uint4);
 }
 int chunk_update_blocks_per_sm(uint32_t d, int block = kChunkBlock);
 // A launch whose rounds give every worker lane at most one update, with chunks of at most
@@ -137,8 +144,12 @@ inline bool chunk_rounds_single(uint64_t flat_len, uint32_t max_chunk, int grid,
 // faster than 1/8 and 1/4), which fits their DictEntry dictionary bytes (32 B x pow2 >= 16 S); the
 // allocation-free entry point uses 8, which fits its fixed array (32 B x pow2 >= 4 S).
 constexpr uint32_t kClaimLoad = 16;
+// Chunks above kClaimMaxChunk run the multi-iteration kernels only, whose many warp-iterations hide a
+// longer probe chain.
+constexpr uint32_t kClaimLoadMulti = 8;
 constexpr uint32_t kClaimLoadNoAlloc = 8;
-inline uint32_t claim_capacity(uint32_t S, uint32_t load = kClaimLoad) {
+inline uint32_t claim_capacity(uint32_t S, uint32_t load = 0) {
+    if (load == 0) load = S > kClaimMaxChunk ? kClaimLoadMulti : kClaimLoad;
     uint64_t need = (uint64_t)load * (uint64_t)S;
     uint64_t cap = 64;
     while (cap < need) cap <<= 1;

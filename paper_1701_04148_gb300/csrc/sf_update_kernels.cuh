@@ -35,6 +35,8 @@ namespace sfk {
 namespace {
 
 constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
+constexpr uint32_t kListSlack = 15u;  // largest slack a claim list entry holds
+constexpr uint32_t kDeleted = 0x80000000u;  // counts of an 8-byte dictionary entry: the key was deleted in the chunk
 
 __device__ __forceinline__ void ld_entry(const DictEntry* ep, unsigned long long& k0, unsigned long long& k1,
                                          unsigned long long& c01, unsigned long long& c23) {
@@ -138,6 +140,62 @@ struct MergeTable {
     uint32_t cd[kSlots];
     ulonglong2 key[kSlots];
 };
+
+// Block-level merge of the warp leaders (lead, ci, cd in place) of one block-iteration; counts the
+// updates and leaders for the next round's choice.  Every thread of the block takes part.
+template <int D, int B>
+__device__ __forceinline__ void merge_block(const LaneWork<D>& L, uint32_t k, bool use_merge, MergeTable<B>& mt,
+                                            uint32_t* s_act, uint32_t* s_lead, uint32_t lane, bool& lead, uint32_t& ci,
+                                            uint32_t& cd) {
+    const unsigned act_b = __ballot_sync(kFull, L.op != 0);
+    const unsigned lead_b = __ballot_sync(kFull, lead);
+    if (lane == 0 && act_b) {
+        atomicAdd(s_act, (uint32_t)__popc(act_b));
+        atomicAdd(s_lead, (uint32_t)__popc(lead_b));
+    }
+    if (!use_merge) return;
+    int role = 0;  // 1: owner of a merge slot, 2: merged into an owner, 3: unmerged
+    uint32_t ms = 0;
+    const uint32_t ftag = ((uint32_t)L.probe ^ (k * 0x9E3779B9u)) | 1u;
+    __syncthreads();
+    if (lead) {
+        ms = (ftag >> 5) & (MergeTable<B>::kSlots - 1);
+        role = 3;
+        for (int p = 0; p < MergeTable<B>::kSlots; ++p) {
+            const uint32_t old = atomicCAS(&mt.tag[ms], 0u, ftag);
+            if (old == 0u) {
+                role = 1;
+                mt.key[ms] = make_ulonglong2(L.k.x0, L.k.x1);
+                mt.run[ms] = k;
+                mt.ci[ms] = ci;
+                mt.cd[ms] = cd;
+                break;
+            }
+            if (old == ftag) {
+                role = 2;
+                break;
+            }
+            ms = (ms + 1) & (MergeTable<B>::kSlots - 1);
+        }
+    }
+    __syncthreads();
+    if (role == 2) {
+        const ulonglong2 o = mt.key[ms];
+        if (o.x == L.k.x0 && o.y == L.k.x1 && mt.run[ms] == k) {
+            atomicAdd(&mt.ci[ms], ci);
+            atomicAdd(&mt.cd[ms], cd);
+            lead = false;
+        } else {
+            role = 3;
+        }
+    }
+    __syncthreads();
+    if (role == 1) {
+        ci = mt.ci[ms];
+        cd = mt.cd[ms];
+        mt.tag[ms] = 0u;  // free for the next block-iteration (after its __syncthreads)
+    }
+}
 
 // What a claiming leader keeps in registers across the barrier (single-iteration rounds): its own
 // counts and the chunk-start minimum m of the key's Slim counters with its minimal-row mask (and,
@@ -260,10 +318,9 @@ __device__ __forceinline__ uint32_t fat_estimate(const SketchDesc& s, const uint
 //          A0_i == m are known from the mask; when c_ins == 1 every other row has A0_i >= m + 1 >= T.
 //   clamp: atomicMin of the bucket bound (maximum, or sum for SF_4) for every row of a deleted key.
 template <int D>
-__device__ __forceinline__ void phase2_key(const SketchDesc& s, uint32_t* ctrl, DictEntry* ep, const uint32_t* h,
-                                           const uint32_t* f, uint32_t c_ins, uint32_t c_del, uint32_t m,
-                                           uint32_t mask, uint32_t F, unsigned long long keep,
-                                           unsigned long long stream) {
+__device__ __forceinline__ void slim_key(const SketchDesc& s, uint32_t* ctrl, const uint32_t* h, const uint32_t* f,
+                                         uint32_t c_ins, bool deleted, uint32_t m, uint32_t mask, uint32_t F,
+                                         unsigned long long keep) {
     if (c_ins) {
         const uint64_t mc = (uint64_t)m + c_ins;
         const uint32_t T = mc < (uint64_t)F ? (uint32_t)mc : F;
@@ -273,13 +330,22 @@ __device__ __forceinline__ void phase2_key(const SketchDesc& s, uint32_t* ctrl, 
                 if (((mask >> i) & 1u) || c_ins > 1u) red_max_pol(slim_ptr(s, i, h[i]), T, keep);
         }
     }
-    if (c_del) {
+    if (deleted) {
         bool under = false;
 #pragma unroll
         for (int i = 0; i < D; ++i)
             red_min_pol(slim_ptr(s, i, h[i]), bucket_bound_cg(s, i, h[i], f[i], &under, keep, true), keep);
         if (under) atomicOr(ctrl + kCtrlErr, kErrUnderflow);
     }
+}
+
+// The same, and the key's entry is cleared.
+template <int D>
+__device__ __forceinline__ void phase2_key(const SketchDesc& s, uint32_t* ctrl, DictEntry* ep, const uint32_t* h,
+                                           const uint32_t* f, uint32_t c_ins, uint32_t c_del, uint32_t m,
+                                           uint32_t mask, uint32_t F, unsigned long long keep,
+                                           unsigned long long stream) {
+    slim_key<D>(s, ctrl, h, f, c_ins, c_del != 0u, m, mask, F, keep);
     asm volatile("st.global.cg.L2::cache_hint.v4.u64 [%0], {%1, %1, %1, %1}, %2;" ::"l"(ep), "l"(0ull), "l"(stream)
                  : "memory");
 }
@@ -299,7 +365,8 @@ template <int D, int B>
 __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_constant__ BatchArgs a) {
     constexpr int kMergeSlots = MergeTable<B>::kSlots;
     extern __shared__ uint2 s_claims_smem[];  // (sketch, dictionary slot) claimed by this block in the round
-    uint2* s_claims = a.claims_global ? a.claims_global + (uint64_t)blockIdx.x * a.claims_cap : s_claims_smem;
+    uint2* s_claims = a.claims_global ? reinterpret_cast<uint2*>(a.claims_global) + (uint64_t)blockIdx.x * a.claims_cap
+                                      : s_claims_smem;
     __shared__ uint32_t s_nclaims;
     __shared__ uint4 s_stage[B / 32][32];
     const SketchRun* runs = a.runs ? a.runs : &a.one;
@@ -313,7 +380,8 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_c
     // every update of the launch is an insertion: Fat counters only grow within a chunk
     const bool ins_only = a.may_ins && !a.may_del;
     uint4* stage = s_stage[threadIdx.x >> 5];
-    unsigned long long target = (a.bar_base + 1ull) * gridDim.x;
+    const unsigned long long per_barrier = (unsigned long long)gridDim.x * a.arrive;
+    unsigned long long target = (a.bar_base + 1ull) * per_barrier;
     // the first flat slot of this warp lies in the same sketch every round
     const uint32_t k_first = gwarp * 32 < a.flat_len ? find_run(runs, a.n_runs, gwarp * 32) : 0u;
 
@@ -376,59 +444,9 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_c
             WarpGroup wg{false, 0u, 0u};
             if (live) wg = warp_group<D>(L, R.s.key_bytes, lane, stage);
 
-            {
-                const unsigned act_b = __ballot_sync(kFull, L.op != 0);
-                const unsigned lead_b = __ballot_sync(kFull, wg.leader);
-                if (lane == 0 && act_b) {
-                    atomicAdd(&s_act, (uint32_t)__popc(act_b));
-                    atomicAdd(&s_lead, (uint32_t)__popc(lead_b));
-                }
-            }
-
-            // block-level merge of equal keys across the block's warps
             bool do_global = wg.leader;
             uint32_t ci = wg.ci, cd = wg.cd;
-            int role = 0;  // 1: owner of a merge slot, 2: merged into an owner, 3: unmerged
-            uint32_t ms = 0;
-            const uint32_t ftag = ((uint32_t)L.probe ^ (k * 0x9E3779B9u)) | 1u;
-            if (use_merge) __syncthreads();
-            if (use_merge && wg.leader) {
-                ms = (ftag >> 5) & (kMergeSlots - 1);
-                role = 3;
-                for (int p = 0; p < kMergeSlots; ++p) {
-                    const uint32_t old = atomicCAS(&s_merge.tag[ms], 0u, ftag);
-                    if (old == 0u) {
-                        role = 1;
-                        s_merge.key[ms] = make_ulonglong2(L.k.x0, L.k.x1);
-                        s_merge.run[ms] = k;
-                        s_merge.ci[ms] = ci;
-                        s_merge.cd[ms] = cd;
-                        break;
-                    }
-                    if (old == ftag) {
-                        role = 2;
-                        break;
-                    }
-                    ms = (ms + 1) & (kMergeSlots - 1);
-                }
-            }
-            if (use_merge) __syncthreads();
-            if (role == 2) {
-                const ulonglong2 o = s_merge.key[ms];
-                if (o.x == L.k.x0 && o.y == L.k.x1 && s_merge.run[ms] == k) {
-                    atomicAdd(&s_merge.ci[ms], ci);
-                    atomicAdd(&s_merge.cd[ms], cd);
-                    do_global = false;
-                } else {
-                    role = 3;
-                }
-            }
-            if (use_merge) __syncthreads();
-            if (role == 1) {
-                ci = s_merge.ci[ms];
-                cd = s_merge.cd[ms];
-                s_merge.tag[ms] = 0u;  // free for the next block-iteration (after its __syncthreads)
-            }
+            merge_block<D, B>(L, k, use_merge, s_merge, &s_act, &s_lead, lane, do_global, ci, cd);
             if (do_global) {
                 OwnCounts own;
                 const uint32_t slot =
@@ -452,8 +470,8 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_c
             }
         }
         have_pre = false;
-        if (!grid_barrier(a.ctrl, target, a.timeout_ns)) return;
-        target += gridDim.x;
+        if (!grid_barrier(a.ctrl, target, a.timeout_ns, a.arrive)) return;
+        target += per_barrier;
 
         // ---- phase 2: Slim raises and clamps, once per distinct key (by its claimer) --------
         if (single) {
@@ -498,7 +516,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_c
 
         // arrive, then prepare the next round's first iteration (keys, ops, hashes) while the
         // other blocks finish, then wait
-        grid_arrive(a.ctrl);
+        grid_arrive(a.ctrl, a.arrive);
         if (r + 1 < a.n_rounds && gwarp * 32 < a.flat_len) {
             const SketchRun& R = runs[k_first];
             const uint64_t o = gwarp * 32 - R.flat_base;
@@ -512,7 +530,193 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_c
             }
         }
         if (!grid_wait(a.ctrl, target, a.timeout_ns)) return;
-        target += gridDim.x;
+        target += per_barrier;
+    }
+}
+
+// ---- multi-iteration rounds with device-resident keys: an 8-byte dictionary ----------------------
+//
+// Same phases as chunk_update_kernel, with less memory behind a distinct key.  Its dictionary entry is 8
+// bytes {claim word, counts}: the claim word is 0x80000000 | 11-bit fingerprint << 20 | position of the
+// claiming update in its chunk (chunks hold at most 2^20), the counts are the key's inserts with bit 31
+// set when it was deleted; one 64-bit CAS claims the entry with the claimer's own counts in it.  A
+// leader whose CAS meets its fingerprint compares its key with the claimer's, read back from the
+// (immutable) key stream, and adds its counts.  The chunk-start minimum and its rows stay with the
+// claimer, in the block's list of claims, and only the claimer reads the Slim.
+template <int D>
+__device__ __forceinline__ bool claim_multi(const SketchRun& R, uint32_t* ctrl, const LaneWork<D>& L, uint64_t base,
+                                            uint32_t pos, uint32_t ci, uint32_t cd, bool may_ins, bool ins_only,
+                                            bool spread, unsigned long long keep, uint4* rec) {
+    const SketchDesc& s = R.s;
+    unsigned long long* E = reinterpret_cast<unsigned long long*>(R.dict);
+    const uint32_t kb = s.key_bytes;
+    const uint32_t claim = 0x80000000u | (uint32_t)(L.probe >> 53) << 20 | pos;
+    const uint32_t counts = ci | (cd ? kDeleted : 0u);
+    const unsigned long long mine = (unsigned long long)counts << 32 | claim;
+    uint32_t slot = (uint32_t)L.probe & R.claim_mask;
+    const int32_t net = (int32_t)ci - (int32_t)cd;
+    uint32_t Fl = 0u;  // 0: no slack (see phase1_global)
+    if (spread && ins_only && ci == 1u) {
+        Fl = 0xFFFFFFFFu;
+#pragma unroll
+        for (int i = 0; i < D; ++i) Fl = min(Fl, atom_add_pol(fat_ptr(s, i, L.h[i], L.f[i]), 1u, keep) + 1u);
+    } else if (net != 0) {
+#pragma unroll
+        for (int i = 0; i < D; ++i) red_add_pol(fat_ptr(s, i, L.h[i], L.f[i]), (uint32_t)net, keep);
+    }
+    // Every leader issues the chunk-start Slim loads ahead of the CAS, though only a claimer uses them: a
+    // load that waits for the CAS waits for a second place in the busy memory system.
+    uint32_t av[D];
+    if (may_ins) {  // no block raises before the barrier
+#pragma unroll
+        for (int i = 0; i < D; ++i) av[i] = ld_cg_pol(slim_ptr(s, i, L.h[i]), keep);
+    }
+    unsigned long long old = atomicCAS(E + slot, 0ull, mine);
+    for (uint32_t p = 0; p <= R.claim_mask; ++p) {
+        if (p > 0u) old = atomicCAS(E + slot, 0ull, mine);
+        if (old == 0ull) {
+            uint32_t m = 0xFFFFFFFFu, ms = 0u;
+            if (may_ins) {
+#pragma unroll
+                for (int i = 0; i < D; ++i) m = min(m, av[i]);
+#pragma unroll
+                for (int i = 0; i < D; ++i) ms |= (av[i] == m ? 1u : 0u) << i;
+                if (ins_only) ms |= min(slack_of(Fl, m), kListSlack) << 8;
+            }
+            *rec = make_uint4(0u, slot, m, ms | pos << 12);
+            return true;
+        }
+        if (((uint32_t)old >> 20) == (claim >> 20)) {
+            const uint64_t t = base + ((uint32_t)old & 0xFFFFFu);
+            const Key o = (kb == 4u || kb == 8u) ? load_key(R.keys, t, kb) : load_key_words(R.keys, R.n * kb, t, kb);
+            if (o.x0 == L.k.x0 && o.x1 == L.k.x1) {
+                uint32_t* c = reinterpret_cast<uint32_t*>(E + slot) + 1;
+                if (ci) atomicAdd(c, ci);
+                if (cd) atomicOr(c, kDeleted);
+                return false;
+            }
+        }
+        slot = (slot + 1u) & R.claim_mask;
+    }
+    atomicOr(ctrl + kCtrlErr, kErrDictFull);
+    return false;
+}
+
+// 1,024 threads per SM at 64 registers (chunk_update_kernel: 512 at 128): the launch waits for memory with
+// no unit busy (at 16 warps per SM L2 39 %, L1 37 %, DRAM 1 % of peak and a fifth of the issue slots
+// used, half of all warp time on loads), so it takes more warps, not fewer instructions.
+template <int D, int B>
+__global__ void __launch_bounds__(B, 1024 / B) chunk_multi_kernel(const __grid_constant__ BatchArgs a) {
+    constexpr int kMergeSlots = MergeTable<B>::kSlots;
+    extern __shared__ uint4 s_list_smem[];  // {sketch, dictionary slot, chunk-start minimum, its rows | slack << 8 | position << 12}
+    uint4* s_list = a.claims_global ? a.claims_global + (uint64_t)blockIdx.x * a.claims_cap : s_list_smem;
+    __shared__ uint32_t s_nclaims;
+    __shared__ uint4 s_stage[B / 32][32];
+    const SketchRun* runs = a.runs ? a.runs : &a.one;
+    const unsigned long long pol_keep = l2_policy_keep();
+    const uint32_t lane = threadIdx.x & 31u;
+    // warps are numbered across blocks first, as in chunk_update_kernel
+    const uint64_t gwarp = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const bool ins_only = a.may_ins && !a.may_del;
+    uint4* stage = s_stage[threadIdx.x >> 5];
+    const unsigned long long per_barrier = (unsigned long long)gridDim.x * a.arrive;
+    unsigned long long target = (a.bar_base + 1ull) * per_barrier;
+    const uint32_t k_first = gwarp * 32 < a.flat_len ? find_run(runs, a.n_runs, gwarp * 32) : 0u;
+
+    __shared__ MergeTable<B> s_merge;
+    for (int i = threadIdx.x; i < kMergeSlots; i += blockDim.x) s_merge.tag[i] = 0u;
+    const uint64_t iters = (a.flat_len + 32 * nwarps - 1) / (32 * nwarps);
+    __shared__ uint32_t s_act, s_lead;
+    __shared__ int s_use_merge;
+    if (threadIdx.x == 0) {
+        s_act = 0u;
+        s_lead = 0u;
+        s_use_merge = 1;
+    }
+
+    for (uint64_t r = 0; r < a.n_rounds; ++r) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_nclaims = 0u;
+            if (r > 0) s_use_merge = (s_act > 0u) && (kMergeRepeats * (s_act - s_lead) >= s_act);
+            s_act = 0u;
+            s_lead = 0u;
+        }
+        __syncthreads();
+        const bool use_merge = s_use_merge != 0;
+
+        // ---- phase 1 ---------------------------------------------------------------------------
+        for (uint64_t it = 0; it < iters; ++it) {
+            const uint64_t j = gwarp * 32 + it * nwarps * 32;
+            LaneWork<D> L;
+            L.op = 0;
+            L.k = Key{0ull, 0ull};
+            L.probe = 0;
+            uint32_t k = 0;
+            bool live = false;
+            if (j < a.flat_len) {
+                k = (it == 0) ? k_first : find_run(runs, a.n_runs, j);
+                const SketchRun& R = runs[k];
+                const uint64_t o = j - R.flat_base;
+                const uint64_t base = r * (uint64_t)R.S;
+                if (base < R.n && o < R.S) {
+                    const uint64_t len = min((uint64_t)R.S, R.n - base);
+                    if (o < len) {
+                        live = true;
+                        prepare<D>(R, a.ctrl, base + o, len - o, lane, stage, L);
+                    }
+                }
+            }
+            const SketchRun& R = runs[k];
+            WarpGroup wg{false, 0u, 0u};
+            if (live) wg = warp_group<D>(L, R.s.key_bytes, lane, stage);
+            bool lead = wg.leader;
+            uint32_t ci = wg.ci, cd = wg.cd;
+            merge_block<D, B>(L, k, use_merge, s_merge, &s_act, &s_lead, lane, lead, ci, cd);
+            if (lead) {
+                const uint64_t base = r * (uint64_t)R.S;
+                uint4 rec;
+                if (claim_multi<D>(R, a.ctrl, L, base, (uint32_t)(j + lane - R.flat_base), ci, cd, a.may_ins != 0, ins_only,
+                                   !use_merge, pol_keep, &rec)) {
+                    rec.x = k;
+                    const uint32_t q = atomicAdd(&s_nclaims, 1u);
+                    if (q < a.claims_cap) s_list[q] = rec;
+                    else atomicOr(a.ctrl + kCtrlErr, kErrDictFull);
+                }
+            }
+        }
+        if (!grid_barrier(a.ctrl, target, a.timeout_ns, a.arrive)) return;
+        target += per_barrier;
+
+        // ---- phase 2: Slim raises and clamps, once per distinct key (by its claimer) --------
+        const uint32_t nclaims = min(s_nclaims, a.claims_cap);
+        for (uint32_t q = threadIdx.x; q < nclaims; q += blockDim.x) {
+            const uint4 rec = s_list[q];
+            const SketchRun& R = runs[rec.x];
+            const uint32_t counts =
+                __ldcg(reinterpret_cast<const uint32_t*>(reinterpret_cast<unsigned long long*>(R.dict) + rec.y) + 1);
+            const uint64_t t = r * (uint64_t)R.S + (rec.w >> 12);
+            const uint32_t kb = R.s.key_bytes;
+            const Key key = (kb == 4u || kb == 8u) ? load_key(R.keys, t, kb) : load_key_words(R.keys, R.n * kb, t, kb);
+            uint32_t h[D], f[D];
+            uint64_t probe;
+            key_indices<D>(R.s, key, h, f, &probe);
+            const uint32_t c_ins = counts & ~kDeleted;
+            const uint32_t F = c_ins ? fat_estimate<D>(R.s, h, f, c_ins, ins_only ? (rec.w >> 8 & kListSlack) : 0u, pol_keep)
+                                     : 0xFFFFFFFFu;
+            slim_key<D>(R.s, a.ctrl, h, f, c_ins, (counts & kDeleted) != 0u, rec.z, rec.w & 0xFFu, F, pol_keep);
+        }
+        // The entries are cleared in a pass of their own: a store right behind the load of the same entry
+        // holds up the memory pipeline (2,530 against 1,884 us on chunks of 200,000).
+        for (uint32_t q = threadIdx.x; q < nclaims; q += blockDim.x) {
+            const uint4 rec = s_list[q];
+            __stcg(reinterpret_cast<uint2*>(reinterpret_cast<unsigned long long*>(runs[rec.x].dict) + rec.y),
+                   make_uint2(0u, 0u));
+        }
+
+        if (!grid_barrier(a.ctrl, target, a.timeout_ns, a.arrive)) return;
+        target += per_barrier;
     }
 }
 
@@ -572,12 +776,12 @@ __device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 1, %0;" 
 // grid_barrier), warps 1.. run work(); the block goes on when both are done.
 template <class Work>
 __device__ __forceinline__ bool grid_barrier_overlapped(uint32_t* ctrl, unsigned long long target, uint64_t timeout_ns,
-                                                        Work&& work) {
+                                                        uint32_t arrive, Work&& work) {
     __shared__ int s_ok_ov;
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned long long* cnt = reinterpret_cast<unsigned long long*>(ctrl + kCtrlBarrier64);
-        red_release_gpu_add_u64(cnt, 1ull);
+        red_release_gpu_add_u64(cnt, arrive);
         int ok = 1;
         if (ld_acquire_gpu_u64(cnt) < target) {
             const uint64_t t0 = globaltimer_ns();
@@ -766,7 +970,8 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
     const uint64_t gwarp = wib ? (uint64_t)(wib - 1) * gridDim.x + blockIdx.x : 0ull;
     uint4* stage = s_stage[wib];
     uint4* stage_ops = s_ops[wib];
-    unsigned long long target = (a.bar_base + 1ull) * gridDim.x;
+    const unsigned long long per_barrier = (unsigned long long)gridDim.x * a.arrive;
+    unsigned long long target = (a.bar_base + 1ull) * per_barrier;
     const uint64_t j = gwarp * 32 + lane;  // this lane's flat slot, the same in every round
     const bool has_slot = wib != 0 && gwarp * 32 < a.flat_len;
     const uint32_t k = has_slot ? find_run(runs, a.n_runs, gwarp * 32) : 0u;
@@ -854,6 +1059,15 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
         claim_key<D>(R, a.ctrl, r * (uint64_t)R.S, (uint32_t)o, dict2 + (r & 1ull) * (R.claim_mask + 1ull), P);
     };
 
+    auto entry_of = [&](uint64_t r, uint32_t slot) { return dict2 + (r & 1ull) * (R.claim_mask + 1ull) + slot; };
+    auto ld_counts = [&](uint64_t r, uint32_t slot) {
+        uint32_t v;
+        asm volatile("ld.global.cg.u32 %0, [%1];"
+                     : "=r"(v)
+                     : "l"(&entry_of(r, slot)->counts));
+        return v;
+    };
+
     if (a.n_rounds == 0) return;
     // chunk 0 is hashed, grouped and claimed before the first round (the counts other leaders add to
     // its entries are read in its phase 2, behind round 0's first barrier); chunk 1 is hashed and
@@ -896,7 +1110,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
         C.slot = P.slot;
         C.m = C.mask = 0u;
         const bool want_m = C.on && (P.ci || a.may_ins);
-        uint32_t av[D];
+        uint32_t av[D], cnt = 0u;
         if (P.lead) {
             const SketchDesc& s = R.s;
             const int32_t net = (int32_t)P.ci - (int32_t)P.cd;
@@ -917,13 +1131,19 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
             }
         }
         // ---- barrier 1; meanwhile the workers claim chunk r + 1 (grouping it first if deferred),
-        // then take the chunk-start minimum and its rows from the loads issued in phase 1 --------
-        if (!grid_barrier_overlapped(a.ctrl, target, a.timeout_ns, [&] {
+        // then read chunk r's other leaders' counts and take the chunk-start minimum and its rows from the
+        // loads issued in phase 1 ------------------------------------------------------------------
+        if (!grid_barrier_overlapped(a.ctrl, target, a.timeout_ns, a.arrive, [&] {
                 if (r + 1 < a.n_rounds) {
                     if (!g_done) group_round(n_live, G);
                     P = G;
                     claim_round(r + 1, P);
                 }
+                // the counts the key's other leaders added, complete since the previous round's second
+                // barrier (chunk 0's only behind this one: read in phase 2).  Read here instead of in
+                // phase 2: 11.7 -> 11.1 us a uniform chunk.  Only the load moves: with the entry's clearing
+                // store right behind it, the pair held up the memory pipeline (37 us).
+                if (C.on && r > 0) cnt = ld_counts(r, C.slot);
                 if (want_m) {
                     uint32_t m = 0xFFFFFFFFu, ms = 0u;
 #pragma unroll
@@ -935,16 +1155,14 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
                 }
             }))
             return;
-        target += gridDim.x;
+        target += per_barrier;
 
-        // ---- phase 2: the key's other leaders' counts, the Fat estimate, Slim raises/clamps --
+        // ---- phase 2: the Fat estimate, Slim raises/clamps, the entry cleared ------------------
         if (C.on) {
             const SketchDesc& s = R.s;
-            ClaimEntry* e = dict2 + (r & 1ull) * (R.claim_mask + 1ull) + C.slot;
-            uint32_t cnt;
-            asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(cnt) : "l"(&e->counts));
+            if (r == 0) cnt = ld_counts(0, C.slot);
             uint32_t F = C.ci ? fat_min<D>(s, C.h, C.f, pol_keep) : 0xFFFFFFFFu;
-            asm volatile("st.global.cg.u64 [%0], %1;" ::"l"(e), "l"(0ull) : "memory");
+            asm volatile("st.global.cg.u64 [%0], %1;" ::"l"(entry_of(r, C.slot)), "l"(0ull) : "memory");
             const uint32_t c_ins = C.ci + (cnt & 0xFFFFu), c_del = C.cd + (cnt >> 16);
             if (c_ins) {
                 if (!C.ci) F = fat_min<D>(s, C.h, C.f, pol_keep);  // only other leaders inserted
@@ -967,7 +1185,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
         }
 
         // ---- barrier 2; meanwhile the workers load, hash and (mostly) group chunk r + 2 ------
-        if (!grid_barrier_overlapped(a.ctrl, target, a.timeout_ns, [&] {
+        if (!grid_barrier_overlapped(a.ctrl, target, a.timeout_ns, a.arrive, [&] {
                 if (r + 2 < a.n_rounds) {
                     fetch_round(r + 2);
                     // the choice needs only the last grouping's counts, so it is taken while the
@@ -982,14 +1200,27 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
                 }
             }))
             return;
-        target += gridDim.x;
+        target += per_barrier;
     }
 }
 
 }  // namespace
 
+// Blocks of the multi-iteration kernel that stay resident for one of the other kernels': 2 when its
+// registers and the claim list let 1,024 threads per SM run.
 template <int D, int B>
-cudaError_t launch_batch_db(const BatchArgs& a, int grid, cudaStream_t st) {
+int multi_blocks(size_t smem) {
+    int nb = 0;
+    if (cudaFuncSetAttribute(chunk_multi_kernel<D, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, chunk_multi_kernel<D, B>, B, smem) != cudaSuccess)
+        return 0;
+    return nb / (kChunkBlock / B);
+}
+
+template <int D, int B>
+cudaError_t launch_batch_db(const BatchArgs& args, int grid, cudaStream_t st) {
+    BatchArgs a = args;
+    a.arrive = kArriveUnits;  // a barrier counts kArriveUnits x grid, whichever kernel passes it
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(B);
@@ -1003,12 +1234,22 @@ cudaError_t launch_batch_db(const BatchArgs& a, int grid, cudaStream_t st) {
         cfg.dynamicSmemBytes = 0;
         return cudaLaunchKernelEx(&cfg, chunk_single_kernel<D, B>, a);
     }
-    const size_t smem = a.claims_global ? 0 : (size_t)a.claims_cap * sizeof(uint2);
-    cudaError_t e = cudaFuncSetAttribute(chunk_update_kernel<D, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    size_t smem = a.claims_global ? 0 : (size_t)a.claims_cap * sizeof(uint4);
+    if (!a.keys_in_host) {
+        const uint32_t cap2 = chunk_claims_cap(a.flat_len, 2 * grid, B);
+        const size_t smem2 = a.claims_global ? 0 : (size_t)cap2 * sizeof(uint4);
+        if (multi_blocks<D, B>(smem2) >= 2) {
+            cfg.gridDim = dim3(2u * (unsigned)grid);
+            a.arrive = kArriveUnits / 2;
+            a.claims_cap = cap2;
+            smem = smem2;
+        }
+    }
+    auto* kernel = a.keys_in_host ? chunk_update_kernel<D, B> : chunk_multi_kernel<D, B>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cfg.dynamicSmemBytes = smem;
-    return cudaLaunchKernelEx(&cfg, chunk_update_kernel<D, B>, a);
+    return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
 template <int D, int B>
