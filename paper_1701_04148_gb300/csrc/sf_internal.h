@@ -144,13 +144,15 @@ inline bool chunk_rounds_single(uint64_t flat_len, uint32_t max_chunk, int grid,
 // faster than 1/8 and 1/4), which fits their DictEntry dictionary bytes (32 B x pow2 >= 16 S); the
 // allocation-free entry point uses 8, which fits its fixed array (32 B x pow2 >= 4 S).
 constexpr uint32_t kClaimLoad = 16;
-// Chunks above kClaimMaxChunk run the multi-iteration kernels only, whose many warp-iterations hide a
-// longer probe chain.
+// Chunks above kClaimMaxChunk run the multi-iteration kernels only, whose warp-iterations hide a longer
+// probe chain: load 8 (chunks of 200,000: 1,626 us a stream against 1,753 at load 4), but at most 2^22
+// entries, 32 MB that L2 holds (chunks of 2^20: 1-2 % faster at load 4 than at 8).
 constexpr uint32_t kClaimLoadMulti = 8;
+constexpr uint64_t kClaimMostMulti = 1ull << 22;
 constexpr uint32_t kClaimLoadNoAlloc = 8;
 inline uint32_t claim_capacity(uint32_t S, uint32_t load = 0) {
-    if (load == 0) load = S > kClaimMaxChunk ? kClaimLoadMulti : kClaimLoad;
-    uint64_t need = (uint64_t)load * (uint64_t)S;
+    uint64_t need = (uint64_t)(load ? load : S > kClaimMaxChunk ? kClaimLoadMulti : kClaimLoad) * (uint64_t)S;
+    if (load == 0 && S > kClaimMaxChunk && need > kClaimMostMulti) need = kClaimMostMulti;
     uint64_t cap = 64;
     while (cap < need) cap <<= 1;
     return (uint32_t)cap;
