@@ -250,7 +250,15 @@ sf_status sf_export_slim(const sf_sketch* s, uint32_t* dst_dev, uint64_t cap_ele
     if (!s || !dst_dev) return SF_ERR_INVALID;
     const uint64_t nelem = (uint64_t)s->p.d * s->p.w;
     if (cap_elems < nelem) return SF_ERR_OOM;
-    if (cudaMemcpyAsync(dst_dev, s->A, nelem * 4ull, cudaMemcpyDeviceToDevice, s->stream) != cudaSuccess)
+    // a kernel copies into memory of the sketch's own device; anything else goes through cudaMemcpyAsync
+    cudaPointerAttributes at{};
+    int cur = -1;
+    const bool own = ((uintptr_t)dst_dev & 3u) == 0 && cudaGetDevice(&cur) == cudaSuccess && cur == s->device &&
+                     cudaPointerGetAttributes(&at, dst_dev) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                     at.device == s->device;
+    if (!own) (void)cudaGetLastError();
+    if ((own ? sfk::launch_copy_counters(s->A, dst_dev, nelem, s->num_sms, s->stream)
+             : cudaMemcpyAsync(dst_dev, s->A, nelem * 4ull, cudaMemcpyDeviceToDevice, s->stream)) != cudaSuccess)
         return SF_ERR_CUDA;
     if (hdr) {
         hdr->magic = SF_SLIM_MAGIC;
@@ -294,11 +302,7 @@ sf_status sf_query_batch(const sf_slim_view* v, const void* keys_dev, uint64_t n
     q.keys = (const uint8_t*)keys_dev;
     q.n = n;
     q.out = out_dev;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return SF_ERR_CUDA;
-    return sfk::launch_query(q, sms, (cudaStream_t)cuda_stream) == cudaSuccess ? SF_OK : SF_ERR_CUDA;
+    return sfk::launch_query(q, (cudaStream_t)cuda_stream) == cudaSuccess ? SF_OK : SF_ERR_CUDA;
 }
 
 sf_status sf_query_pipelined(const sf_slim_view* v, const void* keys_host, uint64_t n, uint32_t* out_host,

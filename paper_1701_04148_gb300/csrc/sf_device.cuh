@@ -213,6 +213,10 @@ __device__ __forceinline__ bool key_equal(const uint8_t* __restrict__ keys, uint
     return o.x0 == k.x0 && o.x1 == k.x1;
 }
 
+// Waits until the kernel before this one in the stream has completed and its writes are visible (a kernel
+// launched with programmatic stream serialization starts before that; otherwise returns at once).
+__device__ __forceinline__ void wait_prior_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -41,6 +41,22 @@ struct BatchArgs {
     int32_t keys_in_host;   // some sketch's keys (or operations) live in host memory, read over the host link
 };
 
+// Launch with programmatic stream serialization: the kernel is launched while the stream's previous kernel
+// drains, and must call wait_prior_kernel before it reads or writes anything.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, ((KArgs)args)...);
+}
+
 inline uint64_t round_up32(uint64_t x) { return (x + 31) & ~31ull; }
 
 // Row seeds of a sketch (the hash reading of sf.h): the first d outputs of SplitMix64 started at
@@ -164,7 +180,9 @@ cudaError_t launch_chunk_update(const SketchRun& one, uint32_t* ctrl, uint64_t b
 // One-at-a-time update (S = 1).
 cudaError_t launch_seq_update(const SeqArgs& a, cudaStream_t st, int smem_limit);
 // Point queries.
-cudaError_t launch_query(const QueryArgs& a, int num_sms, cudaStream_t st);
+cudaError_t launch_query(const QueryArgs& a, cudaStream_t st);
+// Slim export between device buffers.
+cudaError_t launch_copy_counters(const uint32_t* src, uint32_t* dst, uint64_t n, int num_sms, cudaStream_t st);
 cudaError_t launch_multi_query(const MultiQueryArgs& a, int num_sms, cudaStream_t st);
 
 // Dictionary capacity: a power of two >= 16 S for chunks of up to 65,536 updates, >= 8 S above.

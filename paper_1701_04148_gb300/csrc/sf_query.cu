@@ -7,7 +7,7 @@
 // Keys are read per thread, several in flight: one aligned load for 4/8-byte keys, otherwise the
 // aligned 8-byte words covering the key (at most three loads; byte loads only where those words
 // would reach past either end of the caller's buffer).  Measured on 10^6 13-byte keys, back-to-back
-// launches: byte loads 23.0 us, word loads 22.4, word loads with the one-wave grid below 20.8.
+// launches: byte loads 23.0 us, word loads 22.4.
 // Staging a warp's keys through shared memory with 16-byte loads was no faster than byte loads: its
 // byte reads from shared memory meet bank conflicts and cost as many L1 wavefronts.
 #include "sf_internal.h"
@@ -31,6 +31,7 @@ __device__ __forceinline__ Key query_key(const uint8_t* keys, uint64_t total_byt
 template <int D>
 __global__ void __launch_bounds__(kQueryBlock) query_kernel(const QueryArgs q) {
     constexpr int K = kQueryKeys;
+    wait_prior_kernel();
     const SketchDesc& s = q.s;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t t0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t0 < q.n; t0 += K * stride) {
@@ -63,23 +64,16 @@ __global__ void __launch_bounds__(kQueryBlock) query_kernel(const QueryArgs q) {
     }
 }
 
-// The grid is one wave of resident blocks: the 13-byte form holds 40 registers (six blocks per
-// SM), and a fixed eight blocks per SM left a partial second wave (measured: 22.4 -> 20.8 us for
-// 10^6 13-byte keys, 269 -> 256 us for 2^24; capping registers at 32 spilled and ran slower).
+// One iteration per thread: the blocks of a second and third wave start as the first ones' end, where a
+// grid of one resident wave gave every thread two full iterations and some a third, nearly empty one
+// (10^6 13-byte keys 20.0 -> 18.5 us, 4 * 10^6 15-byte keys 28.6 -> 26.7; K = 4 and K = 1 slower).
+// Launched while the stream's previous kernel drains (programmatic stream serialization; the kernel
+// waits for that one's completion before its first access): 18.5 -> 17.1 us, 1,000 keys 4.2 -> 2.3.
 template <int D>
-cudaError_t launch_query_d(const QueryArgs& a, int num_sms, cudaStream_t st) {
-    static int resident = 0;  // blocks per SM, asked once per process and row count
-    if (resident == 0) {
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, query_kernel<D>, kQueryBlock, 0) != cudaSuccess)
-            return cudaGetLastError();
-        resident = nb > 0 ? nb : 1;
-    }
+cudaError_t launch_query_d(const QueryArgs& a, cudaStream_t st) {
     const uint64_t want = (a.n + (uint64_t)kQueryBlock * kQueryKeys - 1) / ((uint64_t)kQueryBlock * kQueryKeys);
-    const uint64_t cap = (uint64_t)num_sms * (uint64_t)resident;
-    const unsigned grid = (unsigned)(want < cap ? want : cap);
-    query_kernel<D><<<grid, kQueryBlock, 0, st>>>(a);
-    return cudaGetLastError();
+    const unsigned grid = (unsigned)(want < 0x7FFFFFFFull ? want : 0x7FFFFFFFull);
+    return launch_overlapped(query_kernel<D>, grid, kQueryBlock, st, a);
 }
 
 // Many requests against many Slims in one launch: thread t answers global slot t, finding its
@@ -114,11 +108,33 @@ __global__ void __launch_bounds__(kQueryBlock) multi_query_kernel(const MultiQue
     }
 }
 
+// Slim export: n counters from src to dst, 16 bytes a thread where both are aligned.
+__global__ void __launch_bounds__(kQueryBlock) copy_counters_kernel(const uint32_t* __restrict__ src,
+                                                                    uint32_t* __restrict__ dst, uint64_t n) {
+    wait_prior_kernel();
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, t0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint64_t done = 0;
+    if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0u) {
+        done = n & ~3ull;
+        for (uint64_t t = t0; t < done / 4; t += stride)
+            reinterpret_cast<uint4*>(dst)[t] = __ldcg(reinterpret_cast<const uint4*>(src) + t);
+    }
+    for (uint64_t t = done + t0; t < n; t += stride) dst[t] = __ldcg(src + t);
+}
+
 }  // namespace
+
+// The counters are copied by a kernel, launched while the update before it drains: a Slim of 64 KiB
+// behind an update takes 1.3 us of the stream's time, cudaMemcpyAsync took 4.1.
+cudaError_t launch_copy_counters(const uint32_t* src, uint32_t* dst, uint64_t n, int num_sms, cudaStream_t st) {
+    if (n == 0) return cudaSuccess;
+    const uint64_t want = (n / 4 + kQueryBlock - 1) / kQueryBlock + 1, cap = (uint64_t)num_sms * 8u;
+    return launch_overlapped(copy_counters_kernel, (unsigned)(want < cap ? want : cap), kQueryBlock, st, src, dst, n);
+}
 
 cudaError_t launch_multi_query(const MultiQueryArgs& a, int num_sms, cudaStream_t st) {
     if (a.total == 0) return cudaSuccess;
-    static int resident = 0;  // one wave of resident blocks, as for query_kernel
+    static int resident = 0;  // one wave of resident blocks
     if (resident == 0) {
         int nb = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, multi_query_kernel, kQueryBlock, 0) != cudaSuccess)
@@ -132,17 +148,17 @@ cudaError_t launch_multi_query(const MultiQueryArgs& a, int num_sms, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t launch_query(const QueryArgs& a, int num_sms, cudaStream_t st) {
+cudaError_t launch_query(const QueryArgs& a, cudaStream_t st) {
     if (a.n == 0) return cudaSuccess;
     switch (a.s.d) {
-        case 1: return launch_query_d<1>(a, num_sms, st);
-        case 2: return launch_query_d<2>(a, num_sms, st);
-        case 3: return launch_query_d<3>(a, num_sms, st);
-        case 4: return launch_query_d<4>(a, num_sms, st);
-        case 5: return launch_query_d<5>(a, num_sms, st);
-        case 6: return launch_query_d<6>(a, num_sms, st);
-        case 7: return launch_query_d<7>(a, num_sms, st);
-        case 8: return launch_query_d<8>(a, num_sms, st);
+        case 1: return launch_query_d<1>(a, st);
+        case 2: return launch_query_d<2>(a, st);
+        case 3: return launch_query_d<3>(a, st);
+        case 4: return launch_query_d<4>(a, st);
+        case 5: return launch_query_d<5>(a, st);
+        case 6: return launch_query_d<6>(a, st);
+        case 7: return launch_query_d<7>(a, st);
+        case 8: return launch_query_d<8>(a, st);
         default: return cudaErrorInvalidValue;
     }
 }
