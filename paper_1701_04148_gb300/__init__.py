@@ -174,6 +174,8 @@ def load_bench(path: str | None = None):
 def load(path: str | None = None):
     """Load the CUDA library (raises if it was not built: there is no CPU path)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             p = path or LIB_PATH
@@ -203,15 +205,26 @@ def check(st: int, what: str) -> int:
     return st
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream_handle(stream=None) -> int:
+    """The stream's handle, by default the current one's (read without building a Stream object: 0.3
+    instead of 2.9 us)."""
+    if stream is not None:
+        return int(stream.cuda_stream)
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return int(torch.cuda.current_stream().cuda_stream)
 
 
 def _dev_ptr(t, what: str) -> int:
@@ -224,13 +237,20 @@ def _dev_ptr(t, what: str) -> int:
     return int(t.data_ptr())
 
 
+_address_of, _byte_at = ctypes.addressof, ctypes.c_char.from_buffer
+
+
 def _host_ptr(a) -> int:
-    """Address of a contiguous host numpy array or CPU tensor (the collector's per-request path:
-    __array_interface__ is about twice as fast as ndarray.ctypes)."""
+    """Address of a contiguous host numpy array or CPU tensor (the collector's per-request path: the
+    buffer protocol takes a third of the time of __array_interface__, which serves the arrays that do
+    not export a writable buffer)."""
     dp = getattr(a, "data_ptr", None)
     if dp is not None:
         return int(dp())
-    return a.__array_interface__["data"][0]
+    try:
+        return _address_of(_byte_at(a))
+    except (TypeError, ValueError, BufferError):
+        return a.__array_interface__["data"][0]
 
 
 def _io_ptr(t, what: str) -> int:
@@ -298,7 +318,7 @@ class Sketch:
 
     def _hold(self, *tensors):
         for t in tensors:
-            if t is not None and t.device.type == "cpu":
+            if t is not None and not t.is_cuda:
                 self._held.append(t)
 
     def reset(self):
@@ -542,7 +562,8 @@ def query(slim, hdr: SlimHeader, keys, out=None, stream=None, index_table=None):
     kb = hdr.key_bytes
     n = keys.shape[0] if (keys.dim() == 2 and keys.dtype == torch.uint8) else keys.numel() * keys.element_size() // kb
     if out is None:
-        out = torch.empty(n, dtype=torch.int32, device=keys.device, pin_memory=not keys.is_cuda)
+        out = torch.empty(n, dtype=torch.int32, device=keys.device) if keys.is_cuda else \
+            torch.empty(n, dtype=torch.int32, pin_memory=True)
     v = SlimView(_dev_ptr(slim, "slim"), hdr, _dev_ptr(index_table, "index_table") if index_table is not None else 0,
                  index_table.shape[0] if index_table is not None else 0)
     check(load().sf_query_batch(ctypes.byref(v), _io_ptr(keys, "keys") if n else 0, n,
@@ -589,6 +610,7 @@ class Collector:
         with torch.cuda.device(self.device):
             check(L.sfc_create(ctypes.byref(cfg), ctypes.byref(h)), "sfc_create")
         self.handle = h
+        self._submit, self._wait = L.sfc_query_submit, L.sfc_wait
         self._live = {}
 
     def upload(self, sketch_id: int, counters, hdr: SlimHeader) -> int:
@@ -604,10 +626,13 @@ class Collector:
         array (or CPU tensor) of one answer per key."""
         t = ctypes.c_uint64()
         n = len(out_np)
-        check(load().sfc_query_submit(self.handle, sketch_id, _host_ptr(keys_np) if n else None, n,
-                                      _host_ptr(out_np) if n else None, ctypes.byref(t)), "sfc_query_submit")
-        self._live[t.value] = (keys_np, out_np)
-        return t.value
+        st = self._submit(self.handle, sketch_id, _host_ptr(keys_np) if n else None, n,
+                          _host_ptr(out_np) if n else None, ctypes.byref(t))
+        if st < 0:
+            raise SFError(st, "sfc_query_submit")
+        ticket = t.value
+        self._live[ticket] = (keys_np, out_np)
+        return ticket
 
     def poll(self, ticket: int) -> int:
         st = load().sfc_poll(self.handle, ticket)
@@ -616,7 +641,7 @@ class Collector:
         return st
 
     def wait(self, ticket: int) -> int:
-        st = load().sfc_wait(self.handle, ticket)
+        st = self._wait(self.handle, ticket)
         self._live.pop(ticket, None)
         return st
 
