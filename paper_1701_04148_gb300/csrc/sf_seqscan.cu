@@ -49,7 +49,9 @@ constexpr uint32_t kDirectBlocks = 16;             // up to here every block sum
 constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr uint32_t kTop = 0xFFFFFFFFu;
 constexpr uint32_t kOpIns = 1u, kOpDel = 2u;       // operation codes of a sorted element (0: none)
+constexpr uint32_t kSlotShift = 19;                // a bucket row's element carries the update's slot above its position
 constexpr uint32_t kHead = 1u << 30, kLast = 1u << 31;
+static_assert(kSeqPiece == 1u << (kSlotShift - 2) && kMaxZ <= 64, "position and slot fit their bits");
 
 // Workspace of one piece.  A sorted element is key << 32 | position << 2 | operation code, so elements
 // compare by (key, position).  Rows 0..d-1 are sorted by bucket, d..2d-1 by Fat counter (bucket x z +
@@ -189,6 +191,11 @@ struct Shared {
         struct {
             uint32_t V[kMaxD][kTile], pos[kMaxD][kTile], low[kMaxD][32];
         } tile;
+        struct {
+            uint32_t at[kMaxD][32][kMaxZ];     // a bucket's counters behind / before a warp's entries
+            uint32_t has[kMaxD][32][2];        // which of them the warp determines
+            uint32_t lanes[32][kMaxZ];         // a warp's lanes by slot
+        } bucket;
     } u;
     uint32_t base[2 * kMaxD + 1][kBins], tot[2 * kMaxD + 1][kBins];
     uint4 warp_agg[kMaxD][32];
@@ -261,7 +268,7 @@ __device__ __forceinline__ bool grid_scan(typename Map::T (&v)[R], typename Map:
     return true;
 }
 
-__device__ __forceinline__ uint32_t el_pos(unsigned long long e) { return ((uint32_t)e >> 2); }
+__device__ __forceinline__ uint32_t el_pos(unsigned long long e) { return (uint32_t)e >> 2 & (kSeqPiece - 1u); }
 __device__ __forceinline__ uint32_t el_op(unsigned long long e) { return (uint32_t)e & 3u; }
 __device__ __forceinline__ uint32_t el_key(unsigned long long e) { return (uint32_t)(e >> 32); }
 
@@ -480,7 +487,7 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
         if (valid) {
 #pragma unroll
             for (int i = 0; i < D; ++i) {
-                w.el0[(uint64_t)i * kSeqPiece + q] = (unsigned long long)h[i] << 32 | pay;
+                w.el0[(uint64_t)i * kSeqPiece + q] = (unsigned long long)h[i] << 32 | f[i] << kSlotShift | pay;
                 w.el0[(uint64_t)(D + i) * kSeqPiece + q] = (unsigned long long)(h[i] * s.z + f[i]) << 32 | pay;
             }
             if constexpr (!kDel) {
@@ -540,60 +547,99 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
         bpo[i] = 0u;
         M[i] = 0u;
         const unsigned long long* Bo = row(i);
-        uint32_t h = 0u;
         if (valid) {
             const unsigned long long e = Bo[q];
-            h = el_key(e);
             bpo[i] = (uint32_t)e;
-            if (q == 0u || el_key(Bo[q - 1u]) != h) bpo[i] |= kHead;
-            if (q + 1u == a.n || el_key(Bo[q + 1u]) != h) bpo[i] |= kLast;
+            if (q == 0u || el_key(Bo[q - 1u]) != el_key(e)) bpo[i] |= kHead;
+            if (q + 1u == a.n || el_key(Bo[q + 1u]) != el_key(e)) bpo[i] |= kLast;
         }
-        if constexpr (!kIns) {
-            // M_i: the bucket's counters right after the deletion, each by a binary search for the last
-            // update on it up to the deletion; a group of lanes takes a deletion, a lane its counters
-            // (the bucket's entries take the same places in both orders, so a bucket that begins and ends
-            // inside this block is searched alone: about 5 steps instead of 17 for 24 entries)
-            const uint32_t gl = s.z <= 4u ? 4u : s.z <= 8u ? 8u : s.z <= 16u ? 16u : 32u;
-            const unsigned long long* C = row(D + i);
+    }
+    if constexpr (!kIns) {
+        // M_i: the bucket's counters right after the deletion, each the value its last update left.  In the
+        // warp that value is a lane's; before the warp it is carried along the block's warps; before the
+        // block it is found by a binary search in the row sorted by counter, once a counter and block;
+        // before the bucket's first update it is the piece's first.  (A search for every deletion and
+        // counter took 50 of 100 us on 100,000 updates with 10,000 deletions.)
+        uint32_t val[D];
+        // the warp's lanes by slot in row i: lanes[k] for slot k
+        auto lanes_by_slot = [&](int i) -> const uint32_t* {
+            uint32_t* tab = sh.u.bucket.lanes[warp];
+            __syncwarp();
+            for (uint32_t k = lane; k < s.z; k += 32u) tab[k] = 0u;
+            __syncwarp();
+            if (valid) atomicOr(&tab[bpo[i] >> kSlotShift & 63u], 1u << lane);
+            __syncwarp();
+            return tab;
+        };
+        auto fat0 = [&](int i, uint32_t key) { return __ldcg(s.B + (uint64_t)i * wz + key); };
+#pragma unroll
+        for (int i = 0; i < D; ++i) {  // the counters of the warp's last bucket behind the warp
+            val[i] = valid ? __ldcg(w.V + (uint64_t)(bpo[i] >> 2 & (kSeqPiece - 1u)) * kStride + i) : 0u;
             const unsigned heads = __ballot_sync(kFull, (bpo[i] & kHead) != 0u);
-            if (lane == 0u) sh.tot[i][warp] = heads;
-            __syncthreads();
-            uint32_t first = 0u, end = a.n;
-            if ((bpo[i] & 3u) == kOpDel) {
-                unsigned b = heads & (kTop >> (31u - lane));
-                int wv = (int)warp;
-                while (!b && wv > 0) b = sh.tot[i][--wv];
-                if (b) first = blk * kTile + (uint32_t)wv * 32u + 31u - (uint32_t)__clz(b);
-                b = lane == 31u ? 0u : heads & (kTop << (lane + 1u));
-                wv = (int)warp;
-                while (!b && wv < 31) b = sh.tot[i][++wv];
-                if (b) end = blk * kTile + (uint32_t)wv * 32u + (uint32_t)__ffs(b) - 1u;
+            const uint32_t* tab = lanes_by_slot(i);
+            const int begin = heads ? 31 - __clz(heads) : -1;  // where that bucket begins, if in this warp
+            const uint32_t h = __shfl_sync(kFull, valid ? el_key(row(i)[q]) : 0u, begin < 0 ? 0 : begin);
+            for (uint32_t k0 = 0; k0 < s.z; k0 += 32u) {
+                const uint32_t k = k0 + lane;
+                const unsigned m = k < s.z ? tab[k] & (begin < 0 ? kFull : kFull << begin) : 0u;
+                uint32_t v = __shfl_sync(kFull, val[i], m ? 31 - __clz(m) : 0);
+                if (!m && begin >= 0 && k < s.z) v = fat0(i, h * s.z + k);
+                const unsigned has = __ballot_sync(kFull, k < s.z && (m || begin >= 0));
+                if (k < s.z) sh.u.bucket.at[i][warp][k] = v;
+                if (lane == 0u) sh.u.bucket.has[i][warp][k0 / 32u] = has;
             }
+        }
+        __syncthreads();
+        if (tid / kMaxZ < (uint32_t)D && tid % kMaxZ < s.z) {  // the counters before each warp
+            const uint32_t i = tid / kMaxZ, k = tid % kMaxZ;
+            const unsigned long long* Bo = row((int)i);
+            const unsigned long long* C = row(D + (int)i);
+            uint32_t carry = 0u;
+            const unsigned long long e = Bo[blk * kTile];
+            if (blk > 0u && el_key(Bo[blk * kTile - 1u]) == el_key(e)) {
+                const uint32_t key = el_key(e) * s.z + k;
+                const unsigned long long want = (unsigned long long)key << 32 | (el_pos(e) << 2);
+                uint32_t lo = 0u, hi = a.n;  // entries below lo are < want, from hi on >= want
+                while (lo < hi) {
+                    const uint32_t mid = (lo + hi) >> 1;
+                    if (C[mid] < want) lo = mid + 1u;
+                    else hi = mid;
+                }
+                carry = lo > 0u && el_key(C[lo - 1u]) == key ? w.Vs[(uint64_t)i * kSeqPiece + lo - 1u] : fat0((int)i, key);
+            }
+#pragma unroll 8
+            for (uint32_t v = 0; v < 32u; ++v) {
+                const uint32_t x = sh.u.bucket.at[i][v][k];
+                sh.u.bucket.at[i][v][k] = carry;
+                if (sh.u.bucket.has[i][v][k / 32u] >> (k % 32u) & 1u) carry = x;
+            }
+        }
+        __syncthreads();
+        // a group of lanes takes a deletion, a lane its counters
+        const uint32_t gl = s.z <= 4u ? 4u : s.z <= 8u ? 8u : s.z <= 16u ? 16u : 32u;
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
             unsigned todo = __ballot_sync(kFull, (bpo[i] & 3u) == kOpDel);
+            if (!todo) continue;
+            const unsigned heads = __ballot_sync(kFull, (bpo[i] & kHead) != 0u);
+            const uint32_t* tab = lanes_by_slot(i);
+            const uint32_t h = valid ? el_key(row(i)[q]) : 0u;
             while (todo) {
                 // the group's deletion: the (lane / gl)-th lane of todo that still waits
                 unsigned rest = todo;
                 for (uint32_t g = 0; g < lane / gl && rest; ++g) rest &= rest - 1u;
-                const int from = rest ? __ffs(rest) - 1 : -1;
-                const uint32_t hd = __shfl_sync(kFull, h, from < 0 ? 0 : from);
-                const uint32_t pd = __shfl_sync(kFull, bpo[i], from < 0 ? 0 : from) & ~(kHead | kLast);
-                const uint32_t f0 = __shfl_sync(kFull, first, from < 0 ? 0 : from);
-                const uint32_t f1 = __shfl_sync(kFull, end, from < 0 ? 0 : from);
+                const int from = rest ? __ffs(rest) - 1 : 0;
+                const uint32_t hd = __shfl_sync(kFull, h, from);
+                const unsigned upto = kFull >> (31 - from), begun = heads & upto;
+                const unsigned span = begun ? upto & (kFull << (31 - __clz(begun))) : upto;
                 uint32_t mx = 0u;
                 uint64_t sum = 0ull;
-                if (from >= 0) {
-                    for (uint32_t k = lane % gl; k < s.z; k += gl) {
-                        const uint32_t key = hd * s.z + k;
-                        const unsigned long long want = (unsigned long long)key << 32 | pd | 3u;
-                        uint32_t lo = f0, hi = f1;  // entries below lo are <= want, from hi on > want
-                        while (lo < hi) {
-                            const uint32_t mid = (lo + hi) >> 1;
-                            if (C[mid] <= want) lo = mid + 1u;
-                            else hi = mid;
-                        }
-                        const bool hit = lo > 0u && el_key(C[lo - 1u]) == key;
-                        const uint32_t v = hit ? w.Vs[(uint64_t)i * kSeqPiece + lo - 1u]
-                                               : __ldcg(s.B + (uint64_t)i * wz + key);
+                for (uint32_t k0 = 0; k0 < s.z; k0 += gl) {
+                    const uint32_t k = k0 + lane % gl;
+                    const unsigned m = k < s.z ? tab[k] & span : 0u;
+                    uint32_t v = __shfl_sync(kFull, val[i], m ? 31 - __clz(m) : 0);
+                    if (k < s.z) {
+                        if (!m) v = begun ? fat0(i, hd * s.z + k) : sh.u.bucket.at[i][warp][k];
                         mx = max(mx, v);
                         sum += v;
                     }
@@ -606,14 +652,13 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
                 // hand the bounds back and strike the deletions taken
                 for (uint32_t g = 0; g < 32u / gl && todo; ++g) {
                     const int at = __ffs(todo) - 1;
-                    const uint32_t b = __shfl_sync(kFull, bound, g * gl);
-                    if ((int)lane == at) M[i] = b;
+                    const uint32_t x = __shfl_sync(kFull, bound, g * gl);
+                    if ((int)lane == at) M[i] = x;
                     todo &= todo - 1u;
                 }
             }
         }
     }
-
     auto least_of = [&](const uint32_t* by_pos, uint32_t pos) {  // minimum over the rows at a position
         uint32_t v[kStride], m = kTop;
         if constexpr (kStride >= 4u) {
@@ -649,7 +694,7 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
             if (bpo[i] & kHead) prev[i].x = __ldcg(slim_ptr(s, i, el_key(row(i)[q])));
         return true;
     };
-    auto pos_of = [&](int i) { return (bpo[i] & ~(kHead | kLast)) >> 2; };
+    auto pos_of = [&](int i) { return bpo[i] >> 2 & (kSeqPiece - 1u); };
     // How many threads of the grid say yes: the words of w.flag rotate over four, and each is cleared two
     // calls before its next use.  One grid barrier; kNone: it gave up.
     uint32_t calls = 0;
