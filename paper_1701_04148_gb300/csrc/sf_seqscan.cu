@@ -18,7 +18,8 @@
 //     every t.  An assignment that an iteration leaves unchanged is therefore the stream-order result.
 //   - From above: T = F everywhere is an upper bound; a scan shows where some row holds less than
 //     T - 1 before the insertion, and T falls to that value plus one.  Sketches whose keys mostly have
-//     one Fat counter to themselves end here at once, or in a few iterations.
+//     one Fat counter to themselves end here at once, or, with the raises along a bucket bounded by their
+//     number (RaiseMap), in a few iterations.
 //   - From below, when that does not end soon: every T at first without any other key's raises.  An
 //     iteration follows a key's own raises along the whole piece: on the row sorted by key,
 //     T_j >= min(F_j, 1 + max(a_j, min(T_{j-1}, G_j))), with a_j the key's Slim minimum of the last
@@ -30,9 +31,10 @@
 // One block of 1,024 threads holds 1,024 consecutive entries of every sorted row, one per thread, in
 // registers across the iterations.  The launch is bound by grid barriers and L2 round trips (about 12
 // barriers when T = F holds), not by bandwidth: its arrays (tens of megabytes at d = 4) stay in L2.
-// Measured on 100,000 Zipf(1) u32 updates (d = 4, w = 4,096, z = 16), a pass: insertions 69 us, where a walk of
-// the stream's dependency graph by one block took 378 us; a tenth of them deletions 121 us, where the
-// window kernel (sf_seq.cu) takes 27.3 ms.
+// Measured on 100,000 Zipf(1) u32 updates (d = 4, w = 4,096, z = 16), a pass, by the stream: insertions 58 to 101 us,
+// where a walk of the stream's dependency graph by one block took 378 to 690; a tenth of them deletions
+// 76 to 114 us, where the window kernel (sf_seq.cu) takes 27.3 ms.  Sorting takes 27 us of it, the Fat 9, the
+// deletions' bounds 12, each scan with its check 8.
 #include "sf_seqscan.h"
 
 namespace sfk {
@@ -64,7 +66,8 @@ struct ScanWs {
     uint32_t* Vs;                   // [d][N] the Fat counter after the update, in counter order
     uint32_t *X, *P;                // [N] the raise target; the previous update of the same key
     uint32_t *hist, *off, *tot;     // digit counts per block (two 16-bit counts a word), first outputs, totals
-    uint4* agg;                     // [d + 1][blocks] block aggregates of a scan
+    uint4* agg;                     // [2d + 1][blocks] block aggregates of the scans (Slim and Fat, keys, raises: a scan
+                                    // may follow one of another kind without a barrier between them)
     uint32_t* low;                  // [d][blocks] least Fat counter of a block's entries in counter order
     uint32_t* flag;                 // [8] "not settled" and "changed" words of the iterations
 };
@@ -95,7 +98,7 @@ __host__ __device__ inline ScanWs carve(void* base, uint32_t d) {
     w.hist = (uint32_t*)take(R * kBlocks * (kBins / 2) * 4);
     w.off = (uint32_t*)take(R * kBlocks * kBins * 4);
     w.tot = (uint32_t*)take(R * kBins * 4);
-    w.agg = (uint4*)take((d + 1) * kBlocks * 16);
+    w.agg = (uint4*)take((2 * d + 1) * kBlocks * 16);
     w.low = (uint32_t*)take(d * kBlocks * 4);
     w.flag = (uint32_t*)take(32);
     return w;
@@ -171,6 +174,29 @@ struct ShiftMap {
     }
     static __device__ __forceinline__ uint4 pack(const T& v) { return make_uint4(v.x, v.y, v.z, 0u); }
     static __device__ __forceinline__ T unpack(const uint4& v) { return make_uint3(v.x, v.y, v.z); }
+};
+
+// Upper bounds along a bucket when an insertion raises by at most one: x -> min(H, max(x, min(x + k, X))), k
+// raises up to the largest of their targets X.  w restarts with the constant H (after a restart z is the
+// value itself).
+struct RaiseMap {
+    using T = uint4;  // {k, X, H, restarted}
+    static __device__ __forceinline__ T identity() { return make_uint4(0u, 0u, kTop, 0u); }
+    static __device__ __forceinline__ T compose(const T& a, const T& b) {
+        if (b.w) return b;
+        const uint32_t up = max(a.z, min(add_sat(a.z, b.x), b.y));
+        return make_uint4(a.x + b.x, max(a.y, b.y), min(b.z, up), a.w);
+    }
+    static __device__ __forceinline__ T shfl_up(const T& v, int o) {
+        return make_uint4(__shfl_up_sync(kFull, v.x, o), __shfl_up_sync(kFull, v.y, o), __shfl_up_sync(kFull, v.z, o),
+                          __shfl_up_sync(kFull, v.w, o));
+    }
+    static __device__ __forceinline__ T shfl_down(const T& v, int o) {
+        return make_uint4(__shfl_down_sync(kFull, v.x, o), __shfl_down_sync(kFull, v.y, o),
+                          __shfl_down_sync(kFull, v.z, o), __shfl_down_sync(kFull, v.w, o));
+    }
+    static __device__ __forceinline__ uint4 pack(const T& v) { return v; }
+    static __device__ __forceinline__ T unpack(const uint4& v) { return v; }
 };
 
 // Inclusive scan of the 32 lanes of a warp.
@@ -249,7 +275,8 @@ __device__ __forceinline__ bool grid_scan(typename Map::T (&v)[R], typename Map:
             // lane 0 holds the composition of all earlier blocks
             const uint4 c0 = Map::pack(c);
             const T carry = Map::unpack(
-                make_uint4(__shfl_sync(kFull, c0.x, 0), __shfl_sync(kFull, c0.y, 0), __shfl_sync(kFull, c0.z, 0), 0u));
+                make_uint4(__shfl_sync(kFull, c0.x, 0), __shfl_sync(kFull, c0.y, 0), __shfl_sync(kFull, c0.z, 0),
+                           __shfl_sync(kFull, c0.w, 0)));
             sh.warp_agg[warp][lane] = Map::pack(Map::compose(carry, Map::unpack(sh.warp_agg[warp][lane])));
         }
     }
@@ -717,27 +744,68 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
     } else {
         // ---- raise targets from above: T = F, lowered where a row holds less than T - 1 ------------------
         if (valid) w.X[q] = least_of(w.V, q);
-        uint32_t most = a.n / 16u;
-        for (uint32_t it = 0;; ++it) {
+        auto lower_where_less = [&](int i, uint32_t before) -> bool {
+            if ((bpo[i] & 3u) != kOpIns || before >= T[i] || before + 1u >= T[i]) return false;
+            atomicMin(w.X + pos_of(i), before + 1u);
+            return true;
+        };
 #pragma unroll
-            for (int i = 0; i < D; ++i)
-                T[i] = (bpo[i] & 3u) != kOpIns ? 0u : it == 0u ? least_of(w.V, pos_of(i)) : __ldcg(w.X + pos_of(i));
-            if (!slim_scan(T)) return;
-            bool lower = false;
+        for (int i = 0; i < D; ++i) T[i] = (bpo[i] & 3u) == kOpIns ? least_of(w.V, pos_of(i)) : 0u;
+        if (!slim_scan(T)) return;
+        bool lower = false;
 #pragma unroll
-            for (int i = 0; i < D; ++i)
-                if ((bpo[i] & 3u) == kOpIns && prev[i].x < T[i] && prev[i].x + 1u < T[i]) {
-                    atomicMin(w.X + pos_of(i), prev[i].x + 1u);
-                    lower = true;
+        for (int i = 0; i < D; ++i) lower |= lower_where_less(i, prev[i].x);
+        uint32_t more = count_of_grid(lower);
+        if (more == kNone) return;
+        settled = more == 0u;
+        if (!settled && 8u * more <= a.n) {
+            // A key whose Fat counters all count other keys too climbs by one an insertion: lowering one T at
+            // a time would take an iteration for each.  So the bounds along a bucket are taken as if an
+            // insertion raised the row's own value by one (T <= a_i + 1 holds in every row), leaving out
+            // the insertions whose T the row holds whatever was raised before (its value under the
+            // clamps alone).  When no T has to fall, T <= m + 1 holds with the raises proper as well.
+            uint32_t hold[D];
+            if constexpr (kIns) {
+#pragma unroll
+                for (int i = 0; i < D; ++i) hold[i] = valid ? __ldcg(slim_ptr(s, i, el_key(row(i)[q]))) : 0u;
+            } else {
+                uint32_t none[D];
+#pragma unroll
+                for (int i = 0; i < D; ++i) none[i] = 0u;
+                if (!slim_scan(none)) return;
+#pragma unroll
+                for (int i = 0; i < D; ++i) hold[i] = prev[i].x;
+            }
+            uint32_t last = more;
+            for (uint32_t it = 1; it <= kAbove; ++it) {
+                uint4 u[D], before[D];
+#pragma unroll
+                for (int i = 0; i < D; ++i) {
+                    const uint32_t op = bpo[i] & 3u;
+                    T[i] = op == kOpIns ? __ldcg(w.X + pos_of(i)) : 0u;
+                    u[i] = RaiseMap::identity();
+                    if (op == kOpIns && T[i] > hold[i]) u[i] = make_uint4(1u, T[i], kTop, 0u);
+                    if (op == kOpDel) u[i].z = M[i];
+                    if (bpo[i] & kHead) {
+                        uint4 start = make_uint4(0u, 0u, __ldcg(slim_ptr(s, i, el_key(row(i)[q]))), 1u);
+                        u[i] = RaiseMap::compose(start, u[i]);
+                    }
                 }
-            const uint32_t more = count_of_grid(lower);
-            if (more == kNone) return;
-            settled = more == 0u;
-            // Go on while the count falls fast: on streams with few coupled keys it falls to a third or less
-            // an iteration, on dense sketches by a tenth.  An iteration takes 8 us at d = 4, the way from
-            // below 20 us before its first one and 12 us for each.
-            if (settled || it == kAbove || (more > 4u && 8u * more > 5u * most)) break;
-            most = more;
+                if (!grid_scan<RaiseMap, D, true>(u, before, sh, w.agg + (uint64_t)(D + 1) * kBlocks, a, target)) return;
+                lower = false;
+#pragma unroll
+                for (int i = 0; i < D; ++i)
+                    lower |= lower_where_less(i, (bpo[i] & kHead) ? __ldcg(slim_ptr(s, i, el_key(row(i)[q]))) : before[i].z);
+                more = count_of_grid(lower);
+                if (more == kNone) return;
+                settled = more == 0u;
+                // three to five iterations settle most streams; where the count does not fall fast the way
+                // from below is shorter (8 us an iteration here; 30 us before the first one there and 15
+                // for each, at d = 4)
+                if (settled || (it >= 3u && 8u * more > 5u * last)) break;
+                last = more;
+            }
+            if (settled && !slim_scan(T)) return;
         }
     }
     if constexpr (!kDel) {
