@@ -314,9 +314,9 @@ __device__ __forceinline__ void cas128(unsigned long long* addr, unsigned long l
 // over what precedes it; the waiter's gpu-scope acquire load that sees the final count, followed
 // by __syncthreads, orders those accesses before every thread's later ones.  A fence.sc on either
 // side adds nothing to this and was measured to cost about 0.2 us per barrier.
-__device__ __forceinline__ void grid_arrive(uint32_t* ctrl, uint32_t arrive = 1u) {
+__device__ __forceinline__ void grid_arrive(uint32_t* ctrl) {
     __syncthreads();
-    if (threadIdx.x == 0) red_release_gpu_add_u64(reinterpret_cast<unsigned long long*>(ctrl + kCtrlBarrier64), arrive);
+    if (threadIdx.x == 0) red_release_gpu_add_u64(reinterpret_cast<unsigned long long*>(ctrl + kCtrlBarrier64), 1ull);
 }
 
 __device__ __forceinline__ bool grid_wait(uint32_t* ctrl, unsigned long long target, uint64_t timeout_ns) {
@@ -340,18 +340,17 @@ __device__ __forceinline__ bool grid_wait(uint32_t* ctrl, unsigned long long tar
     return s_ok_w != 0;
 }
 
-// Grid-wide barrier for a co-resident (cooperatively launched) grid.  Every block adds `arrive` to a
+// Grid-wide barrier for a co-resident (cooperatively launched) grid.  Every block adds 1 to a
 // monotonic 64-bit counter and waits until it reaches `target` = (barriers passed so far + 1) *
-// gridDim.x * arrive.  The wait is bounded: after timeout_ns the block latches kErrTimeout and returns
+// gridDim.x.  The wait is bounded: after timeout_ns the block latches kErrTimeout and returns
 // false, so the kernel leaves instead of hanging.
-__device__ __forceinline__ bool grid_barrier(uint32_t* ctrl, unsigned long long target, uint64_t timeout_ns,
-                                             uint32_t arrive = 1u) {
+__device__ __forceinline__ bool grid_barrier(uint32_t* ctrl, unsigned long long target, uint64_t timeout_ns) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
         unsigned long long* cnt = reinterpret_cast<unsigned long long*>(ctrl + kCtrlBarrier64);
-        red_release_gpu_add_u64(cnt, arrive);
+        red_release_gpu_add_u64(cnt, 1ull);
         if (ld_acquire_gpu_u64(cnt) < target) {
             const uint64_t t0 = globaltimer_ns();
             while (ld_acquire_gpu_u64(cnt) < target) {

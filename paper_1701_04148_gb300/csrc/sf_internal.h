@@ -32,7 +32,6 @@ struct BatchArgs {
     uint64_t n_rounds;      // max over sketches of ceil(n / S)
     uint32_t* ctrl;         // error word + barrier counter
     uint64_t bar_base;      // grid barriers the counter has passed before this launch
-    uint32_t arrive;        // what a block adds to the counter at a barrier (set by the launch)
     uint64_t timeout_ns;
     int32_t may_ins;        // some update of the launch may be an insertion
     int32_t may_del;        // ... a deletion
@@ -117,13 +116,9 @@ constexpr int kChunkBlock = 512;  // default block of the chunked-update kernels
 constexpr int kSeqBlock = 256;
 constexpr int kQueryBlock = 256;
 constexpr uint64_t kBarrierTimeoutNs = 2000000000ull;  // 2 s per wait
-constexpr int kMaxClaimSmem = 112 * 1024;              // dynamic shared memory for the claim list: 7,168 claims of 16
-                                                       // bytes, a block's share of a 2^20-update chunk over 147 SMs or
-                                                       // more; batches keep longer lists in their scratch
-constexpr int kMostClaimSmem = 160 * 1024;             // up to here a launch of one sketch may go: 103 SMs
-// The barrier counter is kept across launches whose grids differ by a factor of two (the multi-iteration
-// kernel runs two blocks where the others run one): a barrier adds kArriveUnits x the smaller grid.
-constexpr uint32_t kArriveUnits = 2;
+// Dynamic shared memory for the claim list: 7,168 claims of 16 bytes (8 in chunk_update_kernel), a block's
+// share of a 2^20-update chunk over 147 SMs or more.  Batches keep longer lists in their scratch.
+constexpr int kMaxClaimSmem = 112 * 1024;
 
 // Chunked update: one cooperative persistent launch per call (one sketch or a batch of sketches
 // sharing d) of `grid` blocks of `block` threads (512, 256 or 128); 2 grid barriers per round.

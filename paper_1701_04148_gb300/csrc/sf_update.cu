@@ -29,7 +29,7 @@ uint32_t chunk_claims_cap(uint64_t flat_len, int grid, int block) {
 }
 
 cudaError_t launch_batch_update(const BatchArgs& a, uint32_t d, int grid, int block, cudaStream_t st) {
-    if (!a.claims_global && (uint64_t)a.claims_cap * sizeof(uint4) > (uint64_t)kMostClaimSmem * block / kChunkBlock)
+    if (!a.claims_global && (uint64_t)a.claims_cap * sizeof(uint2) > (uint64_t)claim_smem_max(block))
         return cudaErrorInvalidValue;
     switch (block) {
         case 512: return launch_batch_block<512>(a, d, grid, st);

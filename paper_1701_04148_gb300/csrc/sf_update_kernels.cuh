@@ -380,8 +380,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_c
     // every update of the launch is an insertion: Fat counters only grow within a chunk
     const bool ins_only = a.may_ins && !a.may_del;
     uint4* stage = s_stage[threadIdx.x >> 5];
-    const unsigned long long per_barrier = (unsigned long long)gridDim.x * a.arrive;
-    unsigned long long target = (a.bar_base + 1ull) * per_barrier;
+    unsigned long long target = (a.bar_base + 1ull) * gridDim.x;
     // the first flat slot of this warp lies in the same sketch every round
     const uint32_t k_first = gwarp * 32 < a.flat_len ? find_run(runs, a.n_runs, gwarp * 32) : 0u;
 
@@ -470,8 +469,8 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_c
             }
         }
         have_pre = false;
-        if (!grid_barrier(a.ctrl, target, a.timeout_ns, a.arrive)) return;
-        target += per_barrier;
+        if (!grid_barrier(a.ctrl, target, a.timeout_ns)) return;
+        target += gridDim.x;
 
         // ---- phase 2: Slim raises and clamps, once per distinct key (by its claimer) --------
         if (single) {
@@ -516,7 +515,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_c
 
         // arrive, then prepare the next round's first iteration (keys, ops, hashes) while the
         // other blocks finish, then wait
-        grid_arrive(a.ctrl, a.arrive);
+        grid_arrive(a.ctrl);
         if (r + 1 < a.n_rounds && gwarp * 32 < a.flat_len) {
             const SketchRun& R = runs[k_first];
             const uint64_t o = gwarp * 32 - R.flat_base;
@@ -530,7 +529,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_update_kernel(const __grid_c
             }
         }
         if (!grid_wait(a.ctrl, target, a.timeout_ns)) return;
-        target += per_barrier;
+        target += gridDim.x;
     }
 }
 
@@ -604,7 +603,10 @@ __device__ __forceinline__ bool claim_multi(const SketchRun& R, uint32_t* ctrl, 
 
 // 1,024 threads per SM at 64 registers (chunk_update_kernel: 512 at 128): the launch waits for memory with
 // no unit busy (at 16 warps per SM L2 39 %, L1 37 %, DRAM 1 % of peak and a fifth of the issue slots
-// used, half of all warp time on loads), so it takes more warps, not fewer instructions.
+// used, half of all warp time on loads), so it takes more warps, not fewer instructions: 32 nodes' sketches
+// 4,350 -> 3,741 us, a 1 GiB Fat 2,060 -> 1,790.  Blocks twice as large as the other kernels' rather than
+// twice as many: the block merge covers more (3,703 -> 3,623 us, chunks of 10^6 3 % faster, of 200,000 2 %
+// slower).
 template <int D, int B>
 __global__ void __launch_bounds__(B, 1024 / B) chunk_multi_kernel(const __grid_constant__ BatchArgs a) {
     constexpr int kMergeSlots = MergeTable<B>::kSlots;
@@ -620,8 +622,7 @@ __global__ void __launch_bounds__(B, 1024 / B) chunk_multi_kernel(const __grid_c
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const bool ins_only = a.may_ins && !a.may_del;
     uint4* stage = s_stage[threadIdx.x >> 5];
-    const unsigned long long per_barrier = (unsigned long long)gridDim.x * a.arrive;
-    unsigned long long target = (a.bar_base + 1ull) * per_barrier;
+    unsigned long long target = (a.bar_base + 1ull) * gridDim.x;
     const uint32_t k_first = gwarp * 32 < a.flat_len ? find_run(runs, a.n_runs, gwarp * 32) : 0u;
 
     __shared__ MergeTable<B> s_merge;
@@ -686,8 +687,8 @@ __global__ void __launch_bounds__(B, 1024 / B) chunk_multi_kernel(const __grid_c
                 }
             }
         }
-        if (!grid_barrier(a.ctrl, target, a.timeout_ns, a.arrive)) return;
-        target += per_barrier;
+        if (!grid_barrier(a.ctrl, target, a.timeout_ns)) return;
+        target += gridDim.x;
 
         // ---- phase 2: Slim raises and clamps, once per distinct key (by its claimer) --------
         const uint32_t nclaims = min(s_nclaims, a.claims_cap);
@@ -715,8 +716,8 @@ __global__ void __launch_bounds__(B, 1024 / B) chunk_multi_kernel(const __grid_c
                    make_uint2(0u, 0u));
         }
 
-        if (!grid_barrier(a.ctrl, target, a.timeout_ns, a.arrive)) return;
-        target += per_barrier;
+        if (!grid_barrier(a.ctrl, target, a.timeout_ns)) return;
+        target += gridDim.x;
     }
 }
 
@@ -776,12 +777,12 @@ __device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 1, %0;" 
 // grid_barrier), warps 1.. run work(); the block goes on when both are done.
 template <class Work>
 __device__ __forceinline__ bool grid_barrier_overlapped(uint32_t* ctrl, unsigned long long target, uint64_t timeout_ns,
-                                                        uint32_t arrive, Work&& work) {
+                                                        Work&& work) {
     __shared__ int s_ok_ov;
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned long long* cnt = reinterpret_cast<unsigned long long*>(ctrl + kCtrlBarrier64);
-        red_release_gpu_add_u64(cnt, arrive);
+        red_release_gpu_add_u64(cnt, 1ull);
         int ok = 1;
         if (ld_acquire_gpu_u64(cnt) < target) {
             const uint64_t t0 = globaltimer_ns();
@@ -970,8 +971,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
     const uint64_t gwarp = wib ? (uint64_t)(wib - 1) * gridDim.x + blockIdx.x : 0ull;
     uint4* stage = s_stage[wib];
     uint4* stage_ops = s_ops[wib];
-    const unsigned long long per_barrier = (unsigned long long)gridDim.x * a.arrive;
-    unsigned long long target = (a.bar_base + 1ull) * per_barrier;
+    unsigned long long target = (a.bar_base + 1ull) * gridDim.x;
     const uint64_t j = gwarp * 32 + lane;  // this lane's flat slot, the same in every round
     const bool has_slot = wib != 0 && gwarp * 32 < a.flat_len;
     const uint32_t k = has_slot ? find_run(runs, a.n_runs, gwarp * 32) : 0u;
@@ -1133,7 +1133,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
         // ---- barrier 1; meanwhile the workers claim chunk r + 1 (grouping it first if deferred),
         // then read chunk r's other leaders' counts and take the chunk-start minimum and its rows from the
         // loads issued in phase 1 ------------------------------------------------------------------
-        if (!grid_barrier_overlapped(a.ctrl, target, a.timeout_ns, a.arrive, [&] {
+        if (!grid_barrier_overlapped(a.ctrl, target, a.timeout_ns, [&] {
                 if (r + 1 < a.n_rounds) {
                     if (!g_done) group_round(n_live, G);
                     P = G;
@@ -1155,7 +1155,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
                 }
             }))
             return;
-        target += per_barrier;
+        target += gridDim.x;
 
         // ---- phase 2: the Fat estimate, Slim raises/clamps, the entry cleared ------------------
         if (C.on) {
@@ -1185,7 +1185,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
         }
 
         // ---- barrier 2; meanwhile the workers load, hash and (mostly) group chunk r + 2 ------
-        if (!grid_barrier_overlapped(a.ctrl, target, a.timeout_ns, a.arrive, [&] {
+        if (!grid_barrier_overlapped(a.ctrl, target, a.timeout_ns, [&] {
                 if (r + 2 < a.n_rounds) {
                     fetch_round(r + 2);
                     // the choice needs only the last grouping's counts, so it is taken while the
@@ -1200,27 +1200,29 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
                 }
             }))
             return;
-        target += per_barrier;
+        target += gridDim.x;
     }
 }
 
 }  // namespace
 
-// Blocks of the multi-iteration kernel that stay resident for one of the other kernels': 2 when its
-// registers and the claim list let 1,024 threads per SM run.
+// Whether the blocks of a chunk_multi_kernel launch, as many as the other kernels' and twice as large, are
+// all resident with a claim list of smem bytes.
 template <int D, int B>
-int multi_blocks(size_t smem) {
+bool multi_fits(size_t smem) {
     int nb = 0;
-    if (cudaFuncSetAttribute(chunk_multi_kernel<D, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, chunk_multi_kernel<D, B>, B, smem) != cudaSuccess)
-        return 0;
-    return nb / (kChunkBlock / B);
+    if (cudaFuncSetAttribute(chunk_multi_kernel<D, 2 * B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, chunk_multi_kernel<D, 2 * B>, 2 * B, smem) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return nb >= kChunkBlock / B;
 }
 
 template <int D, int B>
 cudaError_t launch_batch_db(const BatchArgs& args, int grid, cudaStream_t st) {
     BatchArgs a = args;
-    a.arrive = kArriveUnits;  // a barrier counts kArriveUnits x grid, whichever kernel passes it
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(B);
@@ -1234,26 +1236,25 @@ cudaError_t launch_batch_db(const BatchArgs& args, int grid, cudaStream_t st) {
         cfg.dynamicSmemBytes = 0;
         return cudaLaunchKernelEx(&cfg, chunk_single_kernel<D, B>, a);
     }
-    size_t smem = a.claims_global ? 0 : (size_t)a.claims_cap * sizeof(uint4);
-    // Rounds that give every lane of the smaller grid one update (72,960 to 77,824 slots) stay with
+    // Rounds that give every lane of the smaller blocks one update (72,960 to 77,824 slots) stay with
     // chunk_update_kernel, whose claimers keep their update in registers there: 31 against 35 us for two
     // chunks of 73,161, 236 against 286 for 15 of 71,468.
-    const bool multi = !a.keys_in_host && a.flat_len > (uint64_t)grid * B;
-    if (multi) {
-        const uint32_t cap2 = chunk_claims_cap(a.flat_len, 2 * grid, B);
-        const size_t smem2 = a.claims_global ? 0 : (size_t)cap2 * sizeof(uint4);
-        if (multi_blocks<D, B>(smem2) >= 2) {
-            cfg.gridDim = dim3(2u * (unsigned)grid);
-            a.arrive = kArriveUnits / 2;
-            a.claims_cap = cap2;
-            smem = smem2;
+    if (!a.keys_in_host && a.flat_len > (uint64_t)grid * B) {
+        const uint32_t cap = chunk_claims_cap(a.flat_len, grid, 2 * B);
+        const size_t smem = a.claims_global ? 0 : (size_t)cap * sizeof(uint4);
+        if (multi_fits<D, B>(smem)) {
+            a.claims_cap = cap;
+            cfg.blockDim = dim3(2 * B);
+            cfg.dynamicSmemBytes = smem;
+            return cudaLaunchKernelEx(&cfg, chunk_multi_kernel<D, 2 * B>, a);
         }
     }
-    auto* kernel = multi ? chunk_multi_kernel<D, B> : chunk_update_kernel<D, B>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = a.claims_global ? 0 : (size_t)a.claims_cap * sizeof(uint2);
+    cudaError_t e = cudaFuncSetAttribute(chunk_update_kernel<D, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
     cfg.dynamicSmemBytes = smem;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
+    return cudaLaunchKernelEx(&cfg, chunk_update_kernel<D, B>, a);
 }
 
 template <int D, int B>
