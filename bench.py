@@ -519,7 +519,7 @@ def run_flows(args, ctx):
         # averaged per launch like `achieved`
         fb = tr[rec_key]
         traffic = round(fb["dram_bytes_per_step"] / fb["launches_per_step"])
-    roofline = {"bound": "l2", "kernel": "chunk_update_kernel" if batched else "chunk_single_kernel",
+    roofline = {"bound": "l2", "kernel": "chunk_multi_kernel" if batched else "chunk_single_kernel",
                 "achieved": round(achieved, 2),
                 "peak": round(best["mix"], 2), "unit": "G random L2 ops/s", "frac": round(achieved / best["mix"], 4),
                 "traffic": traffic,
@@ -1066,7 +1066,7 @@ def run_outofl2(args, ctx):
     if tr is not None and "outofl2" in tr:
         rec = tr["outofl2"]
         traffic = round((rec["dram_bytes_read"] + rec["dram_bytes_write"]) / rec["updates"] * n)
-    roofline = {"bound": "hbm", "kernel": "chunk_update_kernel", "achieved": round(achieved, 1),
+    roofline = {"bound": "hbm", "kernel": "chunk_multi_kernel", "achieved": round(achieved, 1),
                 "peak": peaks.get("hbm_gbs"), "unit": "GB/s", "frac": round(achieved / peaks.get("hbm_gbs", 1.0), 4),
                 "traffic": traffic,
                 "counting": f"algorithmic bytes per update: key + op byte + d Fat read-modify-writes "
@@ -1500,7 +1500,7 @@ def run_batch(args, ctx):
     if tr is not None and "c3_group" in tr and info["groups_last"] and tr["c3_group"].get("rounds") == tuned["rounds"]:
         g = tr["c3_group"]
         traffic = round(g["dram_bytes"] / g["updates"] * total / info["groups_last"])
-    roofline = {"bound": "l2", "kernel": "chunk_update_kernel", "achieved": round(ops_s, 2), "peak": round(best["mix"], 2),
+    roofline = {"bound": "l2", "kernel": "chunk_multi_kernel", "achieved": round(ops_s, 2), "peak": round(best["mix"], 2),
                 "unit": "G random L2 ops/s", "frac": round(ops_s / best["mix"], 4),
                 "peak_red_only": round(best["red"], 2), "frac_of_red_only": round(ops_s / best["red"], 4),
                 "peak_load_only": round(best["ld"], 2), "frac_of_load_only": round(ops_s / best["ld"], 4),

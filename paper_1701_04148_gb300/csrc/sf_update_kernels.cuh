@@ -25,6 +25,10 @@
 // T_e <= F_e <= that bound, so the raises and clamps of a
 // counter commute: applying them with atomics in any order gives the stream-order result.
 //
+// Which kernel runs a launch: chunk_single_kernel when every worker lane gets at most one update a round;
+// chunk_multi_kernel for longer rounds with keys in device memory; chunk_update_kernel for keys in host
+// memory (it reads each key once) and rounds of one update per lane that the first does not take.
+//
 // The S = 1 path (the paper's one-at-a-time rule) is in sf_seqscan.cu and sf_seq.cu.
 #pragma once
 

@@ -76,3 +76,27 @@ def test_updates_that_do_nothing(sf):
     for kb in (4, 13):
         k = keys[order] if kb == 4 else torch.cat([keys[order]] * 4, 1)[:, :13]
         _check(sf, 4, 1024, 4, kb, [(k.contiguous(), ops[order].contiguous())])
+
+
+def test_captured_and_replayed(sf):
+    """A captured call replays: the launch leaves the barrier words as it found them."""
+    import torch
+    st, _ = wl.mixed_stream(30_000, 2000, 1.0, 0.1, 4, seed=3)
+    main = torch.cuda.Stream()
+    keys, ops = st.keys.cuda(), st.ops.cuda()
+    torch.cuda.synchronize()
+    g = sf.Sketch(4, 2048, 16, 4, 9, 1, stream=main)
+    o = oracle.Sketch(4, 2048, 16, 4, 9)
+    g.update(keys, ops)
+    o.update(st.keys.numpy(), st.ops.numpy())
+    assert g.sync_status() == sf.SF_OK
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=main):
+        g.update(keys, ops)
+    for _ in range(2):
+        with torch.cuda.stream(main):
+            graph.replay()
+        o.update(st.keys.numpy(), st.ops.numpy())
+    assert g.sync_status() == sf.SF_OK
+    assert np.array_equal(g.fat.cpu().numpy().view(np.uint32).reshape(4, 2048, 16), o.B)
+    assert np.array_equal(g.slim.cpu().numpy().view(np.uint32).reshape(4, 2048), o.A)
