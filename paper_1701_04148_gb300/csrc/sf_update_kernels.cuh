@@ -39,6 +39,7 @@ namespace sfk {
 namespace {
 
 constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
+constexpr uint32_t kSpreadSlots = 32768u;  // rounds above this many slots read two Fat rows first
 constexpr uint32_t kListSlack = 15u;  // largest slack a claim list entry holds
 constexpr uint32_t kDeleted = 0x80000000u;  // counts of an 8-byte dictionary entry: the key was deleted in the chunk
 
@@ -304,6 +305,23 @@ __device__ __forceinline__ uint32_t fat_min(const SketchDesc& s, const uint32_t*
     uint32_t F = 0xFFFFFFFFu;
 #pragma unroll
     for (int i = 0; i < D; ++i) F = min(F, ld_cg_pol(fat_ptr(s, i, h[i], f[i]), keep));
+    return F;
+}
+
+// F_e, or some value of at most m when F_e <= m (the key then raises nothing).  spread: rows 0 and 1 are
+// read first, the others only when both hold more than m, which few keys of a spread-out chunk see.
+template <int D>
+__device__ __forceinline__ uint32_t fat_min_above(const SketchDesc& s, const uint32_t* h, const uint32_t* f, uint32_t m,
+                                                  bool spread, unsigned long long keep) {
+    constexpr int E = D < 2 ? D : 2;
+    if (!spread) return fat_min<D>(s, h, f, keep);
+    uint32_t F = 0xFFFFFFFFu;
+#pragma unroll
+    for (int i = 0; i < E; ++i) F = min(F, ld_cg_pol(fat_ptr(s, i, h[i], f[i]), keep));
+    if (D > E && F > m) {
+#pragma unroll
+        for (int i = E; i < D; ++i) F = min(F, ld_cg_pol(fat_ptr(s, i, h[i], f[i]), keep));
+    }
     return F;
 }
 
@@ -1053,10 +1071,12 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
         s_act = 0u;
         s_lead = 0u;
     };
-    auto group_round = [&](bool live, Pending<D>& G) {
-        workers_sync<B>();
-        if (threadIdx.x == 32) decide();
-        workers_sync<B>();
+    auto group_round = [&](bool live, Pending<D>& G, bool decided = false) {
+        if (!decided) {
+            workers_sync<B>();
+            if (threadIdx.x == 32) decide();
+            workers_sync<B>();
+        }
         group_keys<D, B>(R, live, k, s_use_merge != 0, s_merge, &s_act, &s_lead, lane, stage, G);
     };
     auto claim_round = [&](uint64_t r, Pending<D>& P) {
@@ -1165,7 +1185,12 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
         if (C.on) {
             const SketchDesc& s = R.s;
             if (r == 0) cnt = ld_counts(0, C.slot);
-            uint32_t F = C.ci ? fat_min<D>(s, C.h, C.f, pol_keep) : 0xFFFFFFFFu;
+            // Two Fat rows first where a round's loads queue (long rounds of keys that do not repeat): uniform
+            // chunks of 65,536 11.2 -> 10.7 us, of 50,000 2-4 %, of 32,768 0.4 % faster.  In short or skewed
+            // rounds, and with three rows, the second trip costs more than the loads saved: chunks of
+            // 16,384 5 %, Zipf 1 4 %, d = 3 3 % slower.
+            const bool spread = D >= 4 && a.flat_len > kSpreadSlots && s_use_merge == 0;
+            uint32_t F = C.ci ? fat_min_above<D>(s, C.h, C.f, C.m, spread, pol_keep) : 0xFFFFFFFFu;
             asm volatile("st.global.cg.u64 [%0], %1;" ::"l"(entry_of(r, C.slot)), "l"(0ull) : "memory");
             const uint32_t c_ins = C.ci + (cnt & 0xFFFFu), c_del = C.cd + (cnt >> 16);
             if (c_ins) {
@@ -1196,11 +1221,14 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
                     // copies land (before the hash: 30.97 against 31.06 ms on the single-sketch
                     // sweep, identical counters)
                     workers_sync<B>();
-                    if (threadIdx.x == 32) s_defer = s_act > 0u && (uint64_t)kDeferLeaders * s_lead < (uint64_t)s_act;
+                    if (threadIdx.x == 32) {
+                        s_defer = s_act > 0u && (uint64_t)kDeferLeaders * s_lead < (uint64_t)s_act;
+                        if (!s_defer) decide();  // the merge choice with it (1,433 -> 1,424 us uniform)
+                    }
                     workers_sync<B>();
                     g_done = s_defer == 0;
                     n_live = hash_round(r + 2, G.L);
-                    if (g_done) group_round(n_live, G);
+                    if (g_done) group_round(n_live, G, true);
                 }
             }))
             return;
