@@ -483,6 +483,11 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
     const uint32_t wz = s.w * s.z;
     unsigned long long target = gridDim.x;
     auto barrier = [&]() { return piece_barrier(a, target); };
+    // A launch whose wait gave up leaves the barrier's counter and the count of leaving blocks anywhere, and
+    // every later launch of the stream, until sf_sync zeroes them, would pass its barriers at once and index
+    // with half-written sums.  Such launches do nothing: the error bit stands until sf_sync.  Read ahead of
+    // the hash, whose loads cover its latency.
+    const uint32_t failed = __ldcg(a.ctrl + kCtrlErr) & kErrTimeout;
 
     // ---- hash --------------------------------------------------------------------------------
     {
@@ -525,6 +530,7 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
         }
         if (blk == 0 && tid < 8u) w.flag[tid] = 0u;
     }
+    if (__syncthreads_or((int)failed)) return;
 
     // ---- sort by bucket and by Fat counter -----------------------------------------------------------
     if (!radix_sort<0, 2 * D>(a, w, sh, target, [&](int r) { return r < D ? a.bucket_passes : a.counter_passes; })) return;

@@ -77,3 +77,46 @@ def test_timeout_status_rezeroes_shared_dictionaries_and_the_arena(sf):
     assert bt.sync_status() == sf.SF_OK and e.sync_status() == sf.SF_OK
     assert torch.equal(c.fat, e.fat) and torch.equal(c.slim, e.slim)
     bt.close()
+
+
+@pytest.mark.parametrize("stale", [1, 128, 1 << 40])
+@pytest.mark.parametrize("kind", ["insert", "delete", "mixed"])
+def test_one_at_a_time_launches_after_a_timeout_change_nothing(sf, kind, stale):
+    """The host writes what a one-at-a-time launch that gave up leaves behind: the timeout bit, a barrier
+    count that is not zero and a count of blocks that have left.  The pieces queued behind it (140,000
+    updates: two) must leave every counter as it is; sf_sync reports the timeout and zeroes the words, and
+    the same call then gives the oracle's counters."""
+    import numpy as np
+    import oracle
+    import torch
+    import workloads as wl
+    n = 140_000
+    st, _ = wl.mixed_stream(n, 9000, 1.0, 0.1, 4, seed=12)
+    first, _ = wl.mixed_stream(n, 9000, 1.0, 0.0, 4, seed=12)
+    keys, ops = first.keys.cuda(), None
+    g = sf.Sketch(4, 2048, 16, 4, 9, 1)
+    o = oracle.Sketch(4, 2048, 16, 4, 9)
+    g.insert(keys)
+    o.update(first.keys.numpy(), np.ones(n, np.int8))
+    assert g.sync_status() == sf.SF_OK
+    fat, slim = g.fat.clone(), g.slim.clone()
+    words = g.scratch[:64]                            # the control words
+    words[0] = 2                                      # the timeout bit
+    words[2] = stale & 0x7FFFFFFF                     # the 64-bit barrier count
+    words[3] = stale >> 32
+    words[4] = 1                                      # blocks that have left
+    torch.cuda.synchronize()
+    if kind == "mixed":
+        keys, ops = st.keys.cuda(), st.ops.cuda()
+    call = {"insert": lambda: g.insert(keys), "delete": lambda: g.delete(keys), "mixed": lambda: g.update(keys, ops)}[kind]
+    call()
+    call()
+    assert g.sync_status() == sf.SF_ERR_TIMEOUT
+    assert torch.equal(g.fat, fat) and torch.equal(g.slim, slim)
+    assert int(torch.count_nonzero(g.scratch[:64])) == 0
+    call()
+    op = {"insert": np.ones(n, np.int8), "delete": -np.ones(n, np.int8), "mixed": st.ops.numpy()}[kind]
+    o.update((st.keys if kind == "mixed" else first.keys).numpy(), op)
+    assert g.sync_status() == sf.SF_OK
+    assert np.array_equal(g.fat.cpu().numpy().view(np.uint32).reshape(o.B.shape), o.B)
+    assert np.array_equal(g.slim.cpu().numpy().view(np.uint32).reshape(o.A.shape), o.A)
