@@ -120,3 +120,52 @@ def test_one_at_a_time_launches_after_a_timeout_change_nothing(sf, kind, stale):
     assert g.sync_status() == sf.SF_OK
     assert np.array_equal(g.fat.cpu().numpy().view(np.uint32).reshape(o.B.shape), o.B)
     assert np.array_equal(g.slim.cpu().numpy().view(np.uint32).reshape(o.A.shape), o.A)
+
+
+@pytest.mark.parametrize("chunk", [4096, 100_000])
+@pytest.mark.parametrize("kb", [4, 13])
+def test_stale_claims_past_the_calls_end_are_not_followed(sf, chunk, kb):
+    """A launch that timed out leaves claims of its chunk behind, and the calls made before sf_sync meet them
+    (a batch's next launch runs to its end).  The host plants one in every key's home slot, with the key's
+    fingerprint and a position past the call's last key: the key there is not read, the claim counts as
+    another key's, and the counters equal the oracle's.  Chunks of 4,096 run the single-iteration kernel's
+    dictionary (15-bit fingerprints, 16-bit positions), of 100,000 the multi-iteration one's (11 and 20)."""
+    import numpy as np
+    import oracle
+    import torch
+    U = np.uint64
+
+    def fin(x):
+        x = (x ^ (x >> U(30))) * U(0xBF58476D1CE4E5B9)
+        x = (x ^ (x >> U(27))) * U(0x94D049BB133111EB)
+        return x ^ (x >> U(31))
+
+    seed = 9
+    r = np.random.RandomState(3)
+    distinct = r.randint(0, 256, (200, kb)).astype(np.uint8)
+    keys = distinct[r.randint(0, 200, 700)]
+    full = np.zeros((200, 16), np.uint8)
+    full[:, :kb] = distinct
+    with np.errstate(over="ignore"):
+        probe = fin(full.view("<u8")[:, 0] ^ fin(np.array([seed], U) + U(0x9E3779B97F4A7C15)))
+        if kb > 8:
+            probe = fin(probe ^ full.view("<u8")[:, 1])
+    if chunk == 4096:
+        entries = 16 * chunk
+        claims = (U(0x8000) | probe >> U(49)) << U(16) | U(0xFFFF)
+    else:
+        entries = 1 << 20                              # the power of two from 8 * 100,000
+        claims = U(0x80000000) | (probe >> U(53)) << U(20) | U(0xFFFFF)
+    g = sf.Sketch(4, 3001, 16, kb, seed, chunk)
+    slots = torch.from_numpy((probe & U(entries - 1)).astype(np.int64)).cuda()
+    words = torch.from_numpy((claims & U(0xFFFFFFFF)).astype(np.uint32).view(np.int32)).cuda()
+    g.scratch[64 + 2 * slots] = words
+    planted = g.scratch[64 + 2 * slots]
+    torch.cuda.synchronize()
+    g.insert(torch.from_numpy(keys).cuda())
+    assert g.sync_status() == sf.SF_OK
+    o = oracle.Sketch(4, 3001, 16, kb, seed)
+    o.update(keys, np.ones(700, np.int8), S=chunk)
+    assert np.array_equal(g.fat.cpu().numpy().view(np.uint32).reshape(o.B.shape), o.B)
+    assert np.array_equal(g.slim.cpu().numpy().view(np.uint32).reshape(o.A.shape), o.A)
+    assert torch.equal(g.scratch[64 + 2 * slots], planted)  # nobody took or cleared them
