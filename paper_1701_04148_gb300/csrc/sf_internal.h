@@ -131,6 +131,9 @@ int blocks_per_sm_block(uint32_t d);
 // Dynamic shared memory a block may use for its claim list: 112 KiB at 512 threads, in proportion
 // below, so that 512 / block blocks of a launch fit one SM.
 inline int claim_smem_max(int block) { return kMaxClaimSmem * block / kChunkBlock; }
+// The same for chunk_multi_kernel's blocks of 2 * block threads: 128 KiB beside 82 KiB of static shared memory, 8,192
+// claims, a block's share of a 2^20-update chunk over 128 SMs or more.
+inline int claim_smem_max_multi(int block) { return 128 * 1024 / kChunkBlock * block; }
 // Global claim-list bytes a launch over rounds of up to max_round_slots slots may need (any grid <= 1024 blocks).
 inline uint64_t claims_global_bytes(uint64_t max_round_slots) {
     return (max_round_slots + 1024ull * kChunkBlock) * sizeof(uint4);

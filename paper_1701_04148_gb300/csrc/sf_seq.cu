@@ -395,8 +395,10 @@ cudaError_t launch_seq_update(const SeqArgs& a, cudaStream_t st, int smem_limit)
     if (slim_bytes + fa.sharedSizeBytes <= (uint64_t)smem_limit) {
         b.slim_in_smem = 1;
         smem = (size_t)slim_bytes;
+        // the largest the kernel may ever use: the same value in every call, so that a narrower sketch's
+        // call on another thread does not lower it ahead of this launch
         cudaError_t e = cudaFuncSetAttribute(seq_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+                                             smem_limit - (int)fa.sharedSizeBytes);
         if (e != cudaSuccess) return e;
     }
     seq_update_kernel<<<1, kSeqBlock, smem, st>>>(b);

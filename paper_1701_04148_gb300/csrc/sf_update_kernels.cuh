@@ -1246,12 +1246,14 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
 }  // namespace
 
 // Whether the blocks of a chunk_multi_kernel launch, as many as the other kernels' and twice as large, are
-// all resident with a claim list of smem bytes.
+// all resident with a claim list of smem bytes.  A kernel's largest dynamic shared memory is state of the whole
+// process: every call sets the same value, so a call of another thread never lowers it ahead of a launch.
 template <int D, int B>
 bool multi_fits(size_t smem) {
     int nb = 0;
-    if (cudaFuncSetAttribute(chunk_multi_kernel<D, 2 * B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess ||
+    if (smem > (size_t)claim_smem_max_multi(B) ||
+        cudaFuncSetAttribute(chunk_multi_kernel<D, 2 * B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             claim_smem_max_multi(B)) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, chunk_multi_kernel<D, 2 * B>, 2 * B, smem) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
@@ -1290,7 +1292,7 @@ cudaError_t launch_batch_db(const BatchArgs& args, int grid, cudaStream_t st) {
     }
     const size_t smem = a.claims_global ? 0 : (size_t)a.claims_cap * sizeof(uint2);
     cudaError_t e = cudaFuncSetAttribute(chunk_update_kernel<D, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         claim_smem_max(B));
     if (e != cudaSuccess) return e;
     cfg.dynamicSmemBytes = smem;
     return cudaLaunchKernelEx(&cfg, chunk_update_kernel<D, B>, a);
