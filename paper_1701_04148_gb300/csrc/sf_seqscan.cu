@@ -37,6 +37,8 @@
 // deletions' bounds 12, each scan with its check 8.
 #include "sf_seqscan.h"
 
+#include <type_traits>
+
 namespace sfk {
 
 namespace {
@@ -708,9 +710,11 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
     };
 
     // Slim counters along the bucket orders with raise targets T[i] of this thread's entries: v[i].x after
-    // an entry, prev[i].x before it.
+    // an entry, prev[i].x before it (want_prev).  The read behind the scan's barrier is for callers that meet another
+    // barrier before the counters after the piece are stored: the last scan asks for v alone, since by then
+    // other blocks store the counters of buckets that begin in this one.
     uint2 v[D], prev[D];
-    auto slim_scan = [&](const uint32_t (&T)[D]) -> bool {
+    auto slim_scan = [&](const uint32_t (&T)[D], auto want_prev) -> bool {
 #pragma unroll
         for (int i = 0; i < D; ++i) {
             const uint32_t op = bpo[i] & 3u;
@@ -721,10 +725,13 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
                 v[i] = make_uint2(x, x);
             }
         }
-        if (!grid_scan<ClampMap, D, true>(v, prev, sh, w.agg, a, target)) return false;
+        constexpr bool kPrev = decltype(want_prev)::value;
+        if (!grid_scan<ClampMap, D, kPrev>(v, prev, sh, w.agg, a, target)) return false;
+        if constexpr (kPrev) {
 #pragma unroll
-        for (int i = 0; i < D; ++i)
-            if (bpo[i] & kHead) prev[i].x = __ldcg(slim_ptr(s, i, el_key(row(i)[q])));
+            for (int i = 0; i < D; ++i)
+                if (bpo[i] & kHead) prev[i].x = __ldcg(slim_ptr(s, i, el_key(row(i)[q])));
+        }
         return true;
     };
     auto pos_of = [&](int i) { return bpo[i] >> 2 & (kSeqPiece - 1u); };
@@ -746,7 +753,7 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
     if constexpr (kDel) {
 #pragma unroll
         for (int i = 0; i < D; ++i) T[i] = 0u;
-        if (!slim_scan(T)) return;
+        if (!slim_scan(T, std::false_type{})) return;
     } else {
         // ---- raise targets from above: T = F, lowered where a row holds less than T - 1 ------------------
         if (valid) w.X[q] = least_of(w.V, q);
@@ -757,7 +764,7 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
         };
 #pragma unroll
         for (int i = 0; i < D; ++i) T[i] = (bpo[i] & 3u) == kOpIns ? least_of(w.V, pos_of(i)) : 0u;
-        if (!slim_scan(T)) return;
+        if (!slim_scan(T, std::true_type{})) return;
         bool lower = false;
 #pragma unroll
         for (int i = 0; i < D; ++i) lower |= lower_where_less(i, prev[i].x);
@@ -778,7 +785,7 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
                 uint32_t none[D];
 #pragma unroll
                 for (int i = 0; i < D; ++i) none[i] = 0u;
-                if (!slim_scan(none)) return;
+                if (!slim_scan(none, std::true_type{})) return;
 #pragma unroll
                 for (int i = 0; i < D; ++i) hold[i] = prev[i].x;
             }
@@ -811,7 +818,7 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
                 if (settled || (it >= 3u && 8u * more > 5u * last)) break;
                 last = more;
             }
-            if (settled && !slim_scan(T)) return;
+            if (settled && !slim_scan(T, std::false_type{})) return;
         }
     }
     if constexpr (!kDel) {
@@ -895,7 +902,7 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
 #pragma unroll
                 for (int i = 0; i < D; ++i)
                     T[i] = (bpo[i] & 3u) == kOpIns && it > 0u ? __ldcg(w.X + pos_of(i)) : 0u;
-                if (!slim_scan(T)) return;
+                if (!slim_scan(T, std::true_type{})) return;
 #pragma unroll
                 for (int i = 0; i < D; ++i)
                     if ((bpo[i] & 3u) == kOpIns) w.a[(uint64_t)pos_of(i) * kStride + i] = prev[i].x;
