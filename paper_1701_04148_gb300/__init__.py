@@ -577,7 +577,7 @@ def query(slim, hdr: SlimHeader, keys, out=None, stream=None, index_table=None):
     n = keys.shape[0] if (keys.dim() == 2 and keys.dtype == torch.uint8) else keys.numel() * keys.element_size() // kb
     if out is None:
         out = torch.empty(n, dtype=torch.int32, device=keys.device) if keys.is_cuda else \
-            torch.empty(n, dtype=torch.int32, pin_memory=True)
+            torch.empty(n, dtype=torch.int32, device="cpu", pin_memory=True)
     v = SlimView(_dev_ptr(slim, "slim"), hdr, _dev_ptr(index_table, "index_table") if index_table is not None else 0,
                  index_table.shape[0] if index_table is not None else 0)
     check(load().sf_query_batch(ctypes.byref(v), _io_ptr(keys, "keys") if n else 0, n,
