@@ -25,8 +25,13 @@
 //     T_j >= min(F_j, 1 + max(a_j, min(T_{j-1}, G_j))), with a_j the key's Slim minimum of the last
 //     iteration and G_j a lower bound of the key's Fat minimum between its updates j - 1 and j (every
 //     clamp M_i in between is at least that).  These maps compose as well (a shift and a clamp), so
-//     this is one more segmented scan.  Dense sketches (z = 1, tens of updates per bucket) take tens of
-//     such iterations; each settles at least the first insertion that is not settled yet.
+//     this is one more segmented scan.  Up to four rows, the scan along a bucket also lets each insertion whose
+//     least counter lies there raise whatever it finds by one, as far as its other rows' bounds and F allow
+//     (ClimbMap): keys that take turns in a bucket climb together, where one iteration a turn was needed.
+//     Dense sketches (z = 1, tens of updates per bucket) take 10 to 55 iterations, 11 to 13 us each at d = 2; each
+//     settles at least the first insertion that is not settled yet.  100,000 insertions, w = 1,024, z = 1, by
+//     the stream: d = 2 740-1,455 us without ClimbMap, 255-710 with it; d = 3 470-1,125, 275-720; d = 4
+//     450-1,100, 305-780.
 //
 // One block of 1,024 threads holds 1,024 consecutive entries of every sorted row, one per thread, in
 // registers across the iterations.  The launch is bound by grid barriers and L2 round trips (about 12
@@ -201,6 +206,31 @@ struct RaiseMap {
     static __device__ __forceinline__ T unpack(const uint4& v) { return v; }
 };
 
+// Lower bounds along a bucket: x -> max(lo, min(hi, x), min(x + k, X)), a clamp and k raises by one up to X.  Composing
+// keeps the clamp exactly (raised by the raises of lo) and one ramp of raises, that of all of them together:
+// min(x + k, X) of both, the smaller of the possible caps.  What it drops only lowers the bound, and never
+// below the clamps alone.
+struct ClimbMap {
+    using T = uint4;  // {lo, hi, k, X}; k = 0: no raises
+    static __device__ __forceinline__ T identity() { return make_uint4(0u, kTop, 0u, 0u); }
+    static __device__ __forceinline__ T compose(const T& a, const T& b) {
+        T r;
+        r.x = max(b.x, min(b.y, a.x));
+        r.y = max(b.x, min(b.y, a.y));
+        r.z = a.z + b.z;
+        r.w = min(a.w, b.y);
+        if (b.z) {
+            r.x = max(r.x, min(add_sat(a.x, b.z), b.w));
+            r.w = min(add_sat(a.z ? a.w : a.y, b.z), b.w);
+        }
+        return r;
+    }
+    static __device__ __forceinline__ T shfl_up(const T& v, int o) { return RaiseMap::shfl_up(v, o); }
+    static __device__ __forceinline__ T shfl_down(const T& v, int o) { return RaiseMap::shfl_down(v, o); }
+    static __device__ __forceinline__ uint4 pack(const T& v) { return v; }
+    static __device__ __forceinline__ T unpack(const uint4& v) { return v; }
+};
+
 // Inclusive scan of the 32 lanes of a warp.
 template <class Map>
 __device__ __forceinline__ typename Map::T warp_scan(typename Map::T v, uint32_t lane) {
@@ -242,11 +272,12 @@ __device__ __forceinline__ bool piece_barrier(const ScanArgs& a, unsigned long l
 }
 
 // Scan over R rows at once of the whole grid's entries (one per thread and row): v[r] in, the composition
-// of every entry up to and including this one out; prev[r] (if wanted) without it.  One grid barrier.
-// False: the barrier gave up.
+// of every entry up to and including this one out; prev[r] (if wanted) without it.  One grid barrier, or none
+// when `last` is given: the earlier blocks' part is then what they wrote there at the scan before, with a barrier
+// since.  False: the barrier gave up.
 template <class Map, int R, bool kPrev>
 __device__ __forceinline__ bool grid_scan(typename Map::T (&v)[R], typename Map::T (&prev)[R], Shared& sh, uint4* agg,
-                                          const ScanArgs& a, unsigned long long& target) {
+                                          const ScanArgs& a, unsigned long long& target, const uint4* last = nullptr) {
     using T = typename Map::T;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -263,14 +294,17 @@ __device__ __forceinline__ bool grid_scan(typename Map::T (&v)[R], typename Map:
         sh.warp_agg[warp][lane] = Map::pack(e);
     }
     if (gridDim.x > 1) {
-        if (!grid_barrier(a.ctrl, target, a.timeout_ns)) return false;
-        target += gridDim.x;
+        if (!last) {
+            if (!grid_barrier(a.ctrl, target, a.timeout_ns)) return false;
+            target += gridDim.x;
+            last = agg;
+        }
         if (warp < (uint32_t)R && blockIdx.x > 0) {
             T c = Map::identity();
 #pragma unroll
             for (uint32_t j = 0; j < kBlocks / 32; ++j) {
                 const uint32_t b = lane * (kBlocks / 32) + j;
-                if (b < blockIdx.x) c = Map::compose(c, Map::unpack(__ldcg(agg + warp * kBlocks + b)));
+                if (b < blockIdx.x) c = Map::compose(c, Map::unpack(__ldcg(last + warp * kBlocks + b)));
             }
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) c = Map::compose(c, Map::shfl_down(c, o));
@@ -475,6 +509,10 @@ __device__ __forceinline__ bool radix_sort(const ScanArgs& a, const ScanWs& w, S
 template <int D, bool kIns, bool kDel>
 __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constant__ ScanArgs a) {
     constexpr uint32_t kStride = row_stride(D);
+    // Bounds from below with the raises along a bucket: fewer iterations (d = 2, w = 1,024, z = 1, warm: 155 down to
+    // 23), but twice a clamp's registers a row: at d = 8 the spills cost up to 1.35x of the time.
+    constexpr bool kClimb = D <= 4;
+    using Low = std::conditional_t<kClimb, ClimbMap, ClampMap>;
     extern __shared__ __align__(16) unsigned char s_raw[];
     Shared& sh = *reinterpret_cast<Shared*>(s_raw);
     const SketchDesc& s = a.s;
@@ -694,19 +732,24 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
             }
         }
     }
-    auto least_of = [&](const uint32_t* by_pos, uint32_t pos) {  // minimum over the rows at a position
-        uint32_t v[kStride], m = kTop;
+    // the rows' values at a position, and their minimum
+    auto read_rows = [&](const uint32_t* by_pos, uint32_t pos, uint32_t (&r)[kStride]) -> uint32_t {
+        uint32_t m = kTop;
         if constexpr (kStride >= 4u) {
 #pragma unroll
             for (uint32_t j = 0; j < kStride; j += 4u)
-                *reinterpret_cast<uint4*>(v + j) = __ldcg(reinterpret_cast<const uint4*>(by_pos + (uint64_t)pos * kStride + j));
+                *reinterpret_cast<uint4*>(r + j) = __ldcg(reinterpret_cast<const uint4*>(by_pos + (uint64_t)pos * kStride + j));
         } else {
 #pragma unroll
-            for (uint32_t j = 0; j < kStride; ++j) v[j] = __ldcg(by_pos + (uint64_t)pos * kStride + j);
+            for (uint32_t j = 0; j < kStride; ++j) r[j] = __ldcg(by_pos + (uint64_t)pos * kStride + j);
         }
 #pragma unroll
-        for (int i = 0; i < D; ++i) m = min(m, v[i]);
+        for (int i = 0; i < D; ++i) m = min(m, r[i]);
         return m;
+    };
+    auto least_of = [&](const uint32_t* by_pos, uint32_t pos) {
+        uint32_t r[kStride];
+        return read_rows(by_pos, pos, r);
     };
 
     // Slim counters along the bucket orders with raise targets T[i] of this thread's entries: v[i].x after
@@ -895,23 +938,61 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
                 }
             }
             const uint32_t kop = kpo & 3u, kpos = (kpo & ~kHead) >> 2;
-            uint32_t F = kTop, G = kTop, x = 0u;
+            // {target, where it may be raised: distance of the cap above it << 3 | row} by position, in the half of
+            // the key row that its sort left
+            uint2* rec = reinterpret_cast<uint2*>(((a.key_passes & 1u) ? w.el0 : w.el1) + (uint64_t)(2 * D) * kSeqPiece);
+            uint32_t F = kTop, G = kTop, start[D], had[D], word = 0u;
+            uint2 mine = make_uint2(0u, 0u);
             if (valid) F = least_of(w.V, kpos);
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                start[i] = (bpo[i] & kHead) ? __ldcg(slim_ptr(s, i, el_key(row(i)[q]))) : 0u;
+                had[i] = 0u;
+            }
             // at most one iteration per update: each settles at least the first unsettled insertion
-            for (uint32_t it = 0; it <= a.n; ++it) {
+            for (uint32_t it = 0; it <= a.n + 1u; ++it) {
+                // the last iteration's count, targets and caps, in one trip
+                const uint32_t more = it > 0u ? __ldcg(w.flag + word) : 1u;
+                typename Low::T u[D], before[D];
 #pragma unroll
-                for (int i = 0; i < D; ++i)
-                    T[i] = (bpo[i] & 3u) == kOpIns && it > 0u ? __ldcg(w.X + pos_of(i)) : 0u;
-                if (!slim_scan(T, std::true_type{})) return;
+                for (int i = 0; i < D; ++i) {
+                    const uint32_t op = bpo[i] & 3u;
+                    u[i] = Low::identity();
+                    if (op == kOpIns && it > 0u) {
+                        const uint2 r = __ldcg(rec + pos_of(i));
+                        u[i].x = r.x;
+                        if constexpr (kClimb) {
+                            if ((r.y & 7u) == (uint32_t)i && r.y > 7u) {
+                                u[i].z = 1u;
+                                u[i].w = r.x + (r.y >> 3);
+                            }
+                        }
+                    }
+                    if (op == kOpDel) u[i].y = M[i];
+                    if (bpo[i] & kHead) {
+                        typename Low::T c = Low::identity();
+                        c.x = c.y = start[i];
+                        u[i] = Low::compose(c, u[i]);
+                    }
+                }
+                if (more == 0u) break;  // the targets are as before the last iteration, so v holds the counters after it
+                if (!grid_scan<Low, D, true>(u, before, sh, w.agg, a, target)) return;
 #pragma unroll
-                for (int i = 0; i < D; ++i)
-                    if ((bpo[i] & 3u) == kOpIns) w.a[(uint64_t)pos_of(i) * kStride + i] = prev[i].x;
+                for (int i = 0; i < D; ++i) {
+                    v[i].x = u[i].x;
+                    const uint32_t b = (bpo[i] & kHead) ? start[i] : before[i].x;
+                    // (kClimb's bounds settle unevenly: most are as the last iteration left them)
+                    if ((bpo[i] & 3u) == kOpIns && (!kClimb || it == 0u || b != had[i]))
+                        w.a[(uint64_t)pos_of(i) * kStride + i] = b;
+                    had[i] = b;
+                }
                 if (!barrier()) return;
                 uint3 f[1], unused[1];
                 f[0] = ShiftMap::identity();
+                uint32_t av[kStride], m = kTop;
                 if (valid) {
                     if (kop == kOpIns) {
-                        const uint32_t m = least_of(w.a, kpos);
+                        m = read_rows(w.a, kpos, av);
                         if constexpr (!kIns)
                             if (it == 0u) G = least_of(w.W, kpos);
                         const uint32_t lo = min(F, add_sat(m, 1u));
@@ -925,16 +1006,40 @@ __global__ void __launch_bounds__(kTile, 1) seq_scan_kernel(const __grid_constan
                         f[0] = make_uint3(0u, min(G, F), 0u);  // a deletion
                     }
                 }
-                if (!grid_scan<ShiftMap, 1, false>(f, unused, sh, w.agg + (uint64_t)D * kBlocks, a, target)) return;
+                // From the fourth iteration on, a key's run enters the next block an iteration late, for a barrier less: a
+                // bound from below all the same.  Streams that settle in three or four would take one more.
+                uint4* runs = w.agg + (uint64_t)(D + (it & 1u)) * kBlocks;
+                const uint4* last_runs = it >= 3u ? w.agg + (uint64_t)(D + (~it & 1u)) * kBlocks : nullptr;
+                if (!grid_scan<ShiftMap, 1, false>(f, unused, sh, runs, a, target, last_runs)) return;
                 bool changed = false;
                 if (valid && kop == kOpIns) {
-                    changed = it == 0u || f[0].x != x;
-                    x = f[0].x;
-                    w.X[kpos] = x;
+                    changed = it == 0u || f[0].x != mine.x;
+                    // In the row that alone holds the least of the key's Slim counters the insertion raises whatever
+                    // is there by one, as far as the other rows' bounds and F allow.
+                    uint2 r = make_uint2(f[0].x, 0u);
+                    if constexpr (kClimb) {
+                        uint32_t at = 0u, others = kTop;
+#pragma unroll
+                        for (int i = 0; i < D; ++i) {
+                            if (av[i] == m) at = i;
+                            uint32_t o = kTop;
+#pragma unroll
+                            for (int j = 0; j < D; ++j)
+                                if (j != i) o = min(o, av[j]);
+                            if (av[i] == m) others = o;
+                        }
+                        const uint32_t cap = min(F, add_sat(others, 1u));
+                        if (cap > r.x) r.y = min(cap - r.x, (1u << 29) - 1u) << 3 | at;
+                    }
+                    if (it == 0u || r.x != mine.x || r.y != mine.y) rec[kpos] = r;
+                    mine = r;
                 }
-                const uint32_t more = count_of_grid(changed);
-                if (more == kNone) return;
-                if (more == 0u) break;  // X is as before this iteration, so v holds the counters after it
+                word = calls & 3u;
+                if (blk == 0u && tid == 0u) w.flag[(calls + 2u) & 3u] = 0u;
+                ++calls;
+                const uint32_t c = (uint32_t)__syncthreads_count(changed);
+                if (c && tid == 0u) atomicAdd(w.flag + word, c);
+                if (!barrier()) return;
             }
         }
     }
