@@ -60,3 +60,24 @@ def test_calls_of_two_shapes_from_two_threads(sf, what, shapes):
             o.update(host[i].numpy(), np.ones(N, np.int8), S=chunk if chunk > 1 else None)
         assert np.array_equal(sk[i].fat.cpu().numpy().view(np.uint32).reshape(o.B.shape), o.B)
         assert np.array_equal(sk[i].slim.cpu().numpy().view(np.uint32).reshape(o.A.shape), o.A)
+
+
+def test_one_at_a_time_calls_on_two_streams(sf):
+    """Cooperative launches of two sketches, of up to 128 blocks each, interleave on two streams."""
+    import torch
+    import workloads as wl
+    n = 150_000
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    st = [wl.mixed_stream(n, 7000, 1.0, f, 4, seed=60 + i)[0] for i, f in enumerate((0.0, 0.2))]
+    keys, ops = [s.keys.cuda() for s in st], [s.ops.cuda() for s in st]
+    torch.cuda.synchronize()
+    sk = [sf.Sketch(4, 3000, 16, 4, 5, 1, stream=s) for s in streams]
+    for part in (slice(0, 60_000), slice(60_000, n)):
+        for i in range(2):
+            sk[i].update(keys[i][part], ops[i][part])
+    for i in range(2):
+        o = oracle.Sketch(4, 3000, 16, 4, 5)
+        o.update(st[i].keys.numpy(), st[i].ops.numpy())
+        assert sk[i].sync_status() == sf.SF_OK
+        assert np.array_equal(sk[i].fat.cpu().numpy().view(np.uint32).reshape(o.B.shape), o.B)
+        assert np.array_equal(sk[i].slim.cpu().numpy().view(np.uint32).reshape(o.A.shape), o.A)
