@@ -16,6 +16,11 @@ import ctypes
 import os
 import threading
 
+try:
+    from numpy import ndarray as _ndarray
+except ImportError:  # torch runs without it; host arrays then are tensors
+    _ndarray = None
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "_build", "libsfgb300.so")
 BENCH_LIB_PATH = os.path.join(_HERE, "_build", "libsfbench.so")
@@ -216,17 +221,6 @@ def _torch():
     return _torch_module
 
 
-_numpy_module = None
-
-
-def _numpy():
-    global _numpy_module
-    if _numpy_module is None:
-        import numpy
-        _numpy_module = numpy
-    return _numpy_module
-
-
 def _stream_handle(stream=None) -> int:
     """The stream's handle, by default the current one's (read without building a Stream object: 0.3
     instead of 2.9 us)."""
@@ -259,7 +253,7 @@ def _host_ptr(a) -> int:
     dp = getattr(a, "data_ptr", None)
     if dp is not None:
         return int(dp())
-    if type(a) is _numpy().ndarray:
+    if type(a) is _ndarray:
         try:
             return _address_of(_byte_at(a))
         except (TypeError, ValueError, BufferError):
