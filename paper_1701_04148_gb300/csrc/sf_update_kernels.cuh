@@ -775,6 +775,7 @@ struct alignas(8) ClaimEntry {
 template <int D>
 struct Pending {
     LaneWork<D> L;
+    uint32_t len;     // updates of the chunk
     uint32_t ci, cd;  // counts of the group this lane carries to global memory (0 if it carries none)
     uint32_t slot;    // dictionary slot this lane claimed, kNoSlot if it claimed none
     bool lead;        // this lane increments the Fat for its group
@@ -916,9 +917,11 @@ __device__ __forceinline__ void claim_key(const SketchRun& R, uint32_t* ctrl, ui
             P.slot = slot;
             return;
         }
-        // (a position past the call's end was left by a launch that timed out, see claim_multi)
-        const uint64_t t = base + (old & 0xFFFFu);
-        if ((old >> 16) == fp && t < R.n) {
+        // A position past the chunk's end was left by a launch that timed out (see claim_multi).  The length comes with
+        // the hash: compared with R.n, which this window would have to load, chunks of u32 keys took 2-3 % longer.
+        const uint32_t at = old & 0xFFFFu;
+        if ((old >> 16) == fp && at < P.len) {
+            const uint64_t t = base + at;
             // same fingerprint: the claimer's key is the update at its stored position of this chunk
             const Key o = (kb == 4u || kb == 8u) ? load_key(R.keys, t, kb) : load_key_words(R.keys, R.n * kb, t, kb);
             if (o.x0 == L.k.x0 && o.x1 == L.k.x1) {
@@ -1033,13 +1036,16 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
         if (R.ops) stage_issue(stage_range(reinterpret_cast<const uint8_t*>(R.ops), R.n, first, nv, 1u), lane, stage_ops);
     };
     // wait for those bytes, then decode and hash the lane's update; true when the lane has one
-    auto hash_round = [&](uint64_t r, LaneWork<D>& L) -> bool {
+    auto hash_round = [&](uint64_t r, Pending<D>& P) -> bool {
+        LaneWork<D>& L = P.L;
+        P.len = 0u;
         L.k = Key{0ull, 0ull};
         L.op = 0;
         L.probe = 0;
         uint64_t first = 0;
         const uint32_t nv = warp_span(r, &first);
         if (nv == 0u) return false;
+        P.len = (uint32_t)min((uint64_t)R.S, R.n - r * (uint64_t)R.S);
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
         L.k = stage_take(stage_range(R.keys, R.n * kb, first, nv, kb), nv, kb, lane, stage);
@@ -1111,12 +1117,12 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
     bool n_live = false, g_done = false;  // g_done is the same in every worker thread of a block
     if (wib != 0) {
         fetch_round(0);
-        const bool live0 = hash_round(0, P.L);
+        const bool live0 = hash_round(0, P);
         group_round(live0, P);  // uses the stage: chunk 1's keys are copied into it after that
         if (a.n_rounds > 1) fetch_round(1);
         claim_round(0, P);
         if (a.n_rounds > 1) {
-            n_live = hash_round(1, G.L);
+            n_live = hash_round(1, G);
             group_round(n_live, G);
             g_done = true;
         }
@@ -1231,7 +1237,7 @@ __global__ void __launch_bounds__(B, 512 / B) chunk_single_kernel(const __grid_c
                     }
                     workers_sync<B>();
                     g_done = s_defer == 0;
-                    n_live = hash_round(r + 2, G.L);
+                    n_live = hash_round(r + 2, G);
                     if (g_done) group_round(n_live, G, true);
                 }
             }))
