@@ -184,7 +184,7 @@ def chunk_kernel_source_sha256():
 
 def traffic_record(name="chunk_single_kernel_traffic.json"):
     """DRAM bytes per update of a chunk kernel from a committed ncu summary (the single-iteration
-    kernel's by default; chunk_update_kernel_traffic.json for the multi-iteration kernel), if the
+    kernel's by default; chunk_multi_kernel_traffic.json for the multi-iteration kernel), if the
     kernel sources have not changed since the counters were taken."""
     p = os.path.join(ROOT, "profiles", name)
     if not os.path.exists(p):
@@ -1061,7 +1061,7 @@ def run_outofl2(args, ctx):
     peaks, psrc = measured_peaks()
     achieved = alg_bytes / (t_upd / 1e3) / 1e9
     peaks_r = hbm_random_peaks(ctx["B"], dev, stream)
-    tr = traffic_record("chunk_update_kernel_traffic.json")
+    tr = traffic_record("chunk_multi_kernel_traffic.json")
     traffic = None
     if tr is not None and "outofl2" in tr:
         rec = tr["outofl2"]
@@ -1493,7 +1493,7 @@ def run_batch(args, ctx):
     # and its algorithmic HBM bytes (key 4 B + op 1 B + 4 B per counter access) against the copy peak
     best = l2_random_peaks(ctx["B"], dev, stream)
     ops_s = total * L2_OPS_PER_UPDATE / (tb / 1e3) / 1e9
-    tr = traffic_record("chunk_update_kernel_traffic.json")
+    tr = traffic_record("chunk_multi_kernel_traffic.json")
     traffic = None
     # the captured group's chunks must be those of the tuned round count (DRAM bytes per update
     # grow with the chunk size: a larger chunk touches more dictionary)
@@ -1506,7 +1506,7 @@ def run_batch(args, ctx):
                 "peak_load_only": round(best["ld"], 2), "frac_of_load_only": round(ops_s / best["ld"], 4),
                 "ops_per_update": L2_OPS_PER_UPDATE, "traffic": traffic,
                 "traffic_note": "DRAM bytes per launch: one launch group's application-replay capture "
-                                "(chunk_update_kernel_traffic.json, c3_group) scaled to this step's updates "
+                                "(chunk_multi_kernel_traffic.json, c3_group) scaled to this step's updates "
                                 "and launch groups",
                 "avg_launch_ms": round(tb / max(1, info["groups_last"]), 4)}
     hbm_b = total * (4 + 1 + L2_OPS_PER_UPDATE * 4)

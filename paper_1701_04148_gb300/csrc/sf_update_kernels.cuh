@@ -751,7 +751,7 @@ __global__ void __launch_bounds__(B, 1024 / B) chunk_multi_kernel(const __grid_c
 // When a round gives every lane at most one update (the chunks of one round fit 32 x the warps of
 // the grid) and no chunk exceeds 65,536 updates, each chunk's key dictionary is built one round
 // early.  While round r waits at its first grid barrier -- the L2 is idle then -- the warps group
-// the already loaded and hashed updates of chunk r+1 (warp match, block merge) and claim its
+// the already loaded and hashed updates of chunk r+1 (by warp, then the block merge) and claim its
 // distinct keys in the other half of the dictionary (the halves alternate by chunk parity).  Phase 1
 // of chunk r+1 then only increments the Fat and reads the chunk-start Slim, and phase 2 collects
 // (and clears) what the key's other leaders added to its entry together with the Fat estimate.  The
@@ -828,8 +828,8 @@ __device__ __forceinline__ bool grid_barrier_overlapped(uint32_t* ctrl, unsigned
     return s_ok_ov != 0;
 }
 
-// Group the updates of one chunk, in place in P (whose L holds the lane's hashed update): the warp
-// match, then the block merge when enabled.  Lanes left as leaders (P.lead) carry their group's
+// Group the updates of one chunk, in place in P (whose L holds the lane's hashed update): by warp
+// (warp_group), then the block merge when enabled.  Lanes left as leaders (P.lead) carry their group's
 // insert and delete counts.  Touches shared memory only, so it may run in either barrier window.
 template <int D, int B>
 __device__ __forceinline__ void group_keys(const SketchRun& R, bool live, uint32_t k, bool use_merge,
