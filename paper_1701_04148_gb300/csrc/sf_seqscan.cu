@@ -34,12 +34,13 @@
 //     450-1,100, 305-780.
 //
 // One block of 1,024 threads holds 1,024 consecutive entries of every sorted row, one per thread, in
-// registers across the iterations.  The launch is bound by grid barriers and L2 round trips (10
-// barriers when T = F holds and a bucket's and a counter's index take two radix passes), not by bandwidth: its arrays (tens of megabytes at d = 4) stay in L2.
+// registers across the iterations.  The launch is bound by grid barriers and L2 round trips (10 barriers
+// when T = F holds and the indices of a row's buckets and counters take two radix passes), not by bandwidth: its
+// arrays (tens of megabytes at d = 4) stay in L2.
 // Measured on 100,000 Zipf(1) u32 updates (d = 4, w = 4,096, z = 16), a pass, by the stream: insertions 58 to 101 us,
 // where a walk of the stream's dependency graph by one block took 378 to 690; a tenth of them deletions
-// 76 to 114 us, where the window kernel (sf_seq.cu) takes 27.3 ms.  Sorting takes 27 us of it, the Fat 9, the
-// deletions' bounds 12, each scan with its check 8.
+// 76 to 114 us, where the window kernel (sf_seq.cu) takes 27.3 ms.  Sorting takes 30 us of it, the Fat 9, the
+// deletions' bounds 12, each scan with its check 8 to 15.
 #include "sf_seqscan.h"
 
 #include <type_traits>
