@@ -136,7 +136,7 @@ const char *sf_status_str(sf_status s);
  *                   dictionary with SF_FLAG_SHARED_DICT: see sf_set_dictionary);
  *                   sketches with chunk == 1, w >= 1024 and w*z < 2^32 also hold the
  *                   one-at-a-time workspace of sorts and scans (12 MiB at d = 1, 18 at 2, 26 at 3,
- *                   31 at 4, 42 at 5, 57 at 8)
+ *                   31 at 4, 42 at 5, 56 at 8)
  * Any output pointer may be NULL.  Returns SF_ERR_INVALID for parameters out of range.
  */
 sf_status sf_required_bytes(const sf_params *p, uint64_t *fat_bytes, uint64_t *slim_bytes,
